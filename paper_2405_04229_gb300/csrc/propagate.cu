@@ -1279,12 +1279,18 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
         WarpSmem& W = reinterpret_cast<WarpSmem*>(smem_raw)[t >> 5];
         const int lane = t & 31;
         const long long n_wtiles = (pp.n + kWTile - 1) / kWTile;
-        auto process_tile = [&](const long long tile) {
-            const long long base = tile * kWTile;
+        // `count` (at most 32) segments from `base` on; of their rounds of 32 bunches, those with
+        // index part mod `parts` (a power of two); part 0 counts the segments and what they emit
+        auto process_tile = [&](const long long base, const int count, const int part, const int parts) {
             bool any_beyond = false;   // a bunch of this tile left to the exact pass
-            const int Kt0 = base + lane < pp.n
-                                ? import_segment<SPH, FL>(W, lane, pp.segs + base + lane, pp, ap, dp, invalid, dropped)
+            unsigned int inv = 0, drp = 0;
+            const int Kt0 = lane < count
+                                ? import_segment<SPH, FL>(W, lane, pp.segs + base + lane, pp, ap, dp, inv, drp)
                                 : 0;
+            if (!TR || part == 0) {
+                invalid += inv;
+                dropped += drp;
+            }
             // The warp takes its segments in order of their ground footprint's distance
             // from the LV3 centre (the frame origin unless the filter is on), so that the
             // bunches of a warp round tend to land together: the telescope cells, histogram
@@ -1366,7 +1372,7 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                         my_emit += (unsigned int)N * (unsigned int)W.bunch[sg];
                     }
                 }
-                emitted += my_emit;
+                if (!TR || part == 0) emitted += my_emit;
                 int ph_incl = my_ph;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -1388,7 +1394,8 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                     }
                     __syncwarp();
                     if constexpr (!EX) {
-                        for (int p = lane; p < wn; p += 32) {
+                        const int skip = TR ? (part - (p0 >> 5)) & (parts - 1) : 0;   // rounds of other parts first
+                        for (int p = 32 * skip + lane; p < wn; p += TR ? 32 * parts : 32) {
                             const unsigned int e = W.map[p];
                             const int qs = (int)(e & ((1u << kQBits) - 1)), ib = (int)(e >> kQBits);
                             const bool bey = bunch<false, SPH, REC, FL, TR, kModeMain, FIX>(W, qs, ib, true, base, pp, ap,
@@ -1456,16 +1463,18 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
             }
             if constexpr (!EX) {   // the exact pass is to visit this tile
                 if (__any_sync(0xffffffffu, any_beyond) && lane == 0)
-                    mark_group(scratch, n_wtiles, pp.tiles_per_bit, (unsigned int)tile / (unsigned int)pp.tiles_per_bit);
+                    mark_group(scratch, n_wtiles, pp.tiles_per_bit, (unsigned int)(base / kWTile) / (unsigned int)pp.tiles_per_bit);
             }
         };
         if constexpr (!EX) {
-            for (;;) {   // dynamic scheduling: warp tiles from the work counter
+            for (;;) {   // dynamic scheduling: warp tiles (or their parts) from the work counter
                 unsigned int wt = 0;
                 if (lane == 0) wt = atomicAdd(tile_ctr, 1u);
-                const long long tile = (long long)__shfl_sync(0xffffffffu, wt, 0);
-                if (tile >= n_wtiles) break;
-                process_tile(tile);
+                wt = __shfl_sync(0xffffffffu, wt, 0);
+                const long long base = (long long)(TR ? wt >> pp.parts_log2 : wt) * pp.tile_segs;
+                if (base >= pp.n) break;
+                const int part = TR ? (int)(wt & ((1u << pp.parts_log2) - 1u)) : 0;
+                process_tile(base, (int)std::min<long long>(pp.tile_segs, pp.n - base), part, 1 << pp.parts_log2);
             }
         } else {
             // the exact pass takes the queued bunches 32 at a time, then the marked groups
@@ -1503,7 +1512,8 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                 if (idx >= n_listed) break;
                 const long long g = (long long)__ldcg(list + idx);
                 const long long t_end = std::min<long long>((g + 1) * pp.tiles_per_bit, n_wtiles);
-                for (long long tile = g * pp.tiles_per_bit; tile < t_end; ++tile) process_tile(tile);
+                for (long long tile = g * pp.tiles_per_bit; tile < t_end; ++tile)
+                    process_tile(tile * kWTile, (int)std::min<long long>(kWTile, pp.n - tile * kWTile), 0, 1);
             }
         }
     } else {
@@ -1760,6 +1770,40 @@ cs_status set_smem_attributes() {
 
 int default_blocks_per_sm(const cs_opts& o) { return o.blocks_per_sm > 0 ? o.blocks_per_sm : (o.surrogate ? 1 : 4); }
 
+// How the launch deals n segments out: the grid of the persistent kernel and, for the exact
+// tracer, the segments of a warp tile and the parts that a tile's bunch rounds are split into.
+//
+// Segments per tile.  A launch of `slots` resident warps ends when its last tile does, about half a
+// tile's time (in proportion to tile / bunch) after the others, and every tile costs a fixed import,
+// sort and scan: tail + fixed cost is smallest at tile ~ sqrt(n bunch / slots).  The factor is from
+// sweeps over 1, 2, .. 32 segments: for 1,000 / 5,003 / 20,000 / 62,500 / 262,144 segments of
+// bunch 1 the best tiles are 1-2 / 2 / 4 / 8 / 8-16 (20.6 / 35.0 / 53.8 / 87.1 / 237 us per launch
+// against 65.6 / 108.9 / 110.6 / 127.2 / 262 us with 32), with bunch 5 from 5,003 on 4 / 8 / 16-32 /
+// 32 (26.8 / 34.8 / 47.2 / 82.9 us against 41.9 / 44.8 / 47.2 / 82.9 us).
+//
+// Parts (the stepper only: a round of bunches then takes ~20 times the tile's own work, so that
+// repeating import and sub-steps in up to 16 warps costs little): enough for eight units per
+// resident warp.  1,000 / 10,000 / 100,000 segments of bunch 5: 0.77 / 0.94 / 3.74 ms against
+// 4.69 / 4.90 / 5.67 ms with whole tiles.
+unsigned int plan_launch(PropParams& pp, size_t n, const cs_opts& o) {
+    const long long blocks = (long long)device_sm_count() * default_blocks_per_sm(o);
+    pp.tile_segs = kWTile;
+    pp.parts_log2 = 0;
+    if (o.surrogate) return (unsigned int)std::max<long long>(1, std::min<long long>(((long long)n + kTile - 1) / kTile, blocks));
+    constexpr int wpb = kThreads / 32;   // warps per block
+    const long long slots = blocks * wpb;
+    if (pp.snell) {
+        const long long tiles = ((long long)n + kWTile - 1) / kWTile;
+        while (pp.parts_log2 < 4 && (tiles << pp.parts_log2) < 8 * slots) ++pp.parts_log2;
+    } else {
+        // (to the nearest power of two; fluorescence emits about a tenth of Cherenkov light's bunches)
+        const double best = sqrt(4.75 * (double)n * o.bunch * (o.emission ? 10.0 : 1.0) / (double)slots);
+        while (pp.tile_segs > 1 && pp.tile_segs > best * 1.42) pp.tile_segs >>= 1;
+    }
+    const long long units = (((long long)n + pp.tile_segs - 1) / pp.tile_segs) << pp.parts_log2;
+    return (unsigned int)std::max<long long>(1, std::min<long long>((units + wpb - 1) / wpb, blocks));
+}
+
 __global__ void philox_kernel(const uint4* ctr, size_t n, uint32_t k0, uint32_t k1, uint4* out) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) {
@@ -1950,9 +1994,7 @@ cs_status launch(const cs_segment* d_segs, size_t n, const cs_atmosphere* atm, c
     set_filters(pp, o, det->p, atm->p);
     cs_status st = set_smem_attributes();
     if (st != CS_OK) return st;
-    const int per_sm = default_blocks_per_sm(o);
-    const long long tiles = ((long long)n + kTile - 1) / kTile;
-    const long long grid = std::min<long long>(tiles, (long long)device_sm_count() * per_sm);
+    const unsigned int grid = plan_launch(pp, n, o);
     pp.tiles_per_bit = 1;
     const long long n_wtiles = (pp.n + kWTile - 1) / kWTile;
     pp.q_cap = queue_cap(n_wtiles, o.exact_queue);
@@ -1961,7 +2003,7 @@ cs_status launch(const cs_segment* d_segs, size_t n, const cs_atmosphere* atm, c
     unsigned int* scratch = nullptr;
     if ((st = scratch_alloc(bytes, stream, &scratch)) != CS_OK) return st;
     CS_CUDA_TRY(cudaMemsetAsync(scratch, 0, scratch_zero_words((pp.n + kWTile - 1) / kWTile, 1) * sizeof(unsigned int), stream));
-    st = launch_kernel((unsigned)grid, stream, pp, atm->p, det->p, op, scratch, o.surrogate, o.tc_poll_limit);
+    st = launch_kernel(grid, stream, pp, atm->p, det->p, op, scratch, o.surrogate, o.tc_poll_limit);
     CS_CUDA_TRY(cudaFreeAsync(scratch, stream));
     return st;
 }
@@ -2171,16 +2213,14 @@ extern "C" cs_status cs_propagate_noalloc(const cs_segment* segs, size_t n, cons
     pp.s_max = (float)o.s_max;
     set_filters(pp, o, det->p, atm->p);
     if ((st = set_smem_attributes()) != CS_OK) return st;
-    const int per_sm = default_blocks_per_sm(o);
-    const long long tiles = ((long long)n + kTile - 1) / kTile;
-    const long long grid = std::min<long long>(tiles, (long long)device_sm_count() * per_sm);
+    const unsigned int grid = plan_launch(pp, n, o);
     const long long n_wtiles = ((long long)n + kWTile - 1) / kWTile;
     pp.tiles_per_bit = (int)std::max<long long>(1, (n_wtiles + kNoAllocBits - 1) / kNoAllocBits);
     pp.q_cap = 0;   // no queue in the fixed array: every bunch beyond the tables marks its group
     pp.q_off = 0;
     // the array keeps the previous call's counters and map: start this call's at zero
     CS_CUDA_TRY(cudaMemsetAsync(ctr, 0, scratch_zero_words(n_wtiles, pp.tiles_per_bit) * sizeof(unsigned int), stream));
-    return launch_kernel((unsigned)grid, stream, pp, atm->p, dp, op, ctr, o.surrogate, o.tc_poll_limit);
+    return launch_kernel(grid, stream, pp, atm->p, dp, op, ctr, o.surrogate, o.tc_poll_limit);
 }
 
 // ---------------------------------------------------------------------------
@@ -2217,22 +2257,11 @@ size_t scratch_bytes(size_t n) {
     return scratch_words(n_wtiles, 1, queue_cap(n_wtiles)) * sizeof(unsigned int);
 }
 
-// Grid of the persistent launch; also sets the kernel's shared-memory limit
-// (host-side calls kept out of stream capture).
-cs_status prepare_launch(size_t n, const cs_opts& o, unsigned int* grid) {
-    cs_status st = set_smem_attributes();
-    if (st != CS_OK) return st;
-    const int per_sm = default_blocks_per_sm(o);
-    const long long tiles = ((long long)n + kTile - 1) / kTile;
-    *grid = (unsigned)std::max<long long>(1, std::min<long long>(tiles, (long long)device_sm_count() * per_sm));
-    return CS_OK;
-}
-
 // Zeroing (unless accumulating), counter reset and the kernel, on `stream`;
 // only stream operations, so it can be captured.
 cs_status enqueue(const cs_segment* segs, size_t n, const cs_atmosphere* atm, const cs_detector* det,
                   uint64_t seed, const int* d_bunch, const cs_opts& o, const cs_output* out, unsigned int* ctr,
-                  unsigned int grid, cudaStream_t stream) {
+                  cudaStream_t stream) {
     const DetParams& dp = det->p;
     const OutParams op = out_params(out);
     if (!o.accumulate) {
@@ -2250,6 +2279,7 @@ cs_status enqueue(const cs_segment* segs, size_t n, const cs_atmosphere* atm, co
     pp.shower_bunch = d_bunch;
     pp.s_max = (float)o.s_max;
     set_filters(pp, o, det->p, atm->p);
+    const unsigned int grid = plan_launch(pp, n, o);
     pp.tiles_per_bit = 1;
     pp.q_cap = std::min(queue_cap(((long long)n + kWTile - 1) / kWTile, o.exact_queue),
                         queue_cap(((long long)n + kWTile - 1) / kWTile));   // within the scratch's default size
@@ -2302,8 +2332,7 @@ extern "C" cs_status cs_batch_create(const cs_segment* segs, size_t n, const cs_
     cudaError_t e;
     if ((e = cudaMalloc(&b->d_ctr, scratch_bytes(n))) != cudaSuccess) { set_last_error("batch scratch", e); return fail(CS_ERR_CUDA); }
     if ((st = upload_bunches(det, shower_bunch, &b->d_bunch)) != CS_OK) return fail(st);
-    unsigned int grid = 1;
-    if ((st = prepare_launch(n, o, &grid)) != CS_OK) return fail(st);
+    if ((st = set_smem_attributes()) != CS_OK) return fail(st);   // kept out of the capture
     if ((e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking)) != cudaSuccess) {
         set_last_error("capture stream", e);
         return fail(CS_ERR_CUDA);
@@ -2312,7 +2341,7 @@ extern "C" cs_status cs_batch_create(const cs_segment* segs, size_t n, const cs_
         set_last_error("begin capture", e);
         return fail(CS_ERR_CUDA);
     }
-    st = enqueue(segs, n, atm, det, seed, b->d_bunch, o, out, b->d_ctr, grid, cap);
+    st = enqueue(segs, n, atm, det, seed, b->d_bunch, o, out, b->d_ctr, cap);
     cudaGraph_t g = nullptr;
     e = cudaStreamEndCapture(cap, &g);
     b->graph = g;
@@ -2373,14 +2402,13 @@ extern "C" cs_status cs_autotune_tiling(const cs_segment* segs, size_t n, const 
     float best = 3.0e38f;
     for (int bpm = 1; bpm <= 4; ++bpm) {
         o.blocks_per_sm = bpm;
-        unsigned int grid = 1;
-        if ((st = prepare_launch(n, o, &grid)) != CS_OK) return done(st);
-        if ((st = enqueue(segs, n, atm, det, seed, d_bunch, o, out, ctr, grid, stream)) != CS_OK) return done(st);
+        if ((st = set_smem_attributes()) != CS_OK) return done(st);
+        if ((st = enqueue(segs, n, atm, det, seed, d_bunch, o, out, ctr, stream)) != CS_OK) return done(st);
         float total = 0.0f;
         for (int r = 0; r < 3; ++r) {
             float ms = 0.0f;
             if ((e = cudaEventRecord(e0, stream)) != cudaSuccess) { set_last_error("tune", e); return done(CS_ERR_CUDA); }
-            if ((st = enqueue(segs, n, atm, det, seed, d_bunch, o, out, ctr, grid, stream)) != CS_OK) return done(st);
+            if ((st = enqueue(segs, n, atm, det, seed, d_bunch, o, out, ctr, stream)) != CS_OK) return done(st);
             if ((e = cudaEventRecord(e1, stream)) != cudaSuccess || (e = cudaEventSynchronize(e1)) != cudaSuccess ||
                 (e = cudaEventElapsedTime(&ms, e0, e1)) != cudaSuccess) {
                 set_last_error("tune timing", e);
@@ -2510,11 +2538,9 @@ extern "C" cs_status cs_streamer_run(cs_streamer* s, const cs_segment* host_segs
     CS_CUDA_TRY(cudaGetDevice(&dev));
     if (dev != s->device) return CS_ERR_INVALID_ARG;
     cudaStream_t stream = (cudaStream_t)stream_;
-    unsigned int grid = 0;
-    st = prepare_launch(std::min(n, s->chunk), o, &grid);
-    if (st != CS_OK) return st;
+    if ((st = set_smem_attributes()) != CS_OK) return st;
     // zeroing (unless accumulating) on the caller's stream, then both streams wait for it
-    st = enqueue(nullptr, 0, atm, det, seed, nullptr, o, out, nullptr, grid, stream);
+    st = enqueue(nullptr, 0, atm, det, seed, nullptr, o, out, nullptr, stream);
     if (st != CS_OK) return st;
     CS_CUDA_TRY(cudaEventRecord(s->ev_in, stream));
     for (int b = 0; b < 2; ++b) CS_CUDA_TRY(cudaStreamWaitEvent(s->st[b], s->ev_in, 0));
@@ -2527,7 +2553,7 @@ extern "C" cs_status cs_streamer_run(cs_streamer* s, const cs_segment* host_segs
         CS_CUDA_TRY(cudaMemcpyAsync(s->d_buf[b], host_segs + off, m * sizeof(cs_segment), cudaMemcpyHostToDevice,
                                     s->st[b]));
         oc.seg_base = o.seg_base + off;
-        st = enqueue(s->d_buf[b], m, atm, det, seed, nullptr, oc, out, s->d_scratch[b], grid, s->st[b]);
+        st = enqueue(s->d_buf[b], m, atm, det, seed, nullptr, oc, out, s->d_scratch[b], s->st[b]);
         if (st != CS_OK) return st;
     }
     // the caller's stream continues after both streams' last chunks
