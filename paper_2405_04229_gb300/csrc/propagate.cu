@@ -63,21 +63,21 @@ struct TileSmem {
 // the block-wide tile above).
 constexpr int kWTile = 32;              // segments per warp tile
 constexpr int kWSubCap = 128;           // sub-steps per warp round
-constexpr int kWMapCap = 256;           // bunches per warp map window
 struct WarpSmem {
     float4 segA[kWTile], segB[kWTile], segC[kWTile], segD[kWTile];   // as in TileSmem
     double t0[kWTile];
     float g[kWTile], z2[kWTile];
     int shower[kWTile];
     int bunch[kWTile];
-    int offK[kWTile + 1];
-    int perm[kWTile];      // tile slot of the i-th segment in processing order
-    float4 sub[kWSubCap];
-    int nsub_ph[kWSubCap];
-    unsigned int map[kWMapCap];
+    float4 sub[kWSubCap];        // the round's sub-steps that emit a bunch, in order
+    int first[kWSubCap + 32];    // index of each one's first bunch, then 32 entries past every bunch
+};
+struct WarpSmemPass : WarpSmem { // the exact pass also queues bunches beyond the tables
+    int q_sub[64], q_bunch[64];
 };
 constexpr size_t kSmemExact = (kThreads / 32) * sizeof(WarpSmem);
-static_assert(4 * (kSmemExact + 1024) <= 228 * 1024, "four exact-tracer blocks per SM");
+constexpr size_t kSmemPass = (kThreads / 32) * sizeof(WarpSmemPass);
+static_assert(4 * (kSmemPass + 1024) <= 228 * 1024, "four exact-tracer blocks per SM");
 
 // The surrogate instances keep the tensor-core network's buffers after the tile.
 constexpr size_t kTcSmemOffset = (sizeof(TileSmem) + 127) & ~(size_t)127;
@@ -302,11 +302,11 @@ __device__ __forceinline__ float fluorescence_line(const PropParams& pp, uint32_
     return fp.fl_inv_l[line];
 }
 
-// Stage 2 (Eq. 2.2-2.5, Sec. 4.2.1): sub-step k of tile segment sg at local
-// slot q: angle and mean bunch count at the sub-step midpoint, stochastic
-// rounding with the sub-step's own draw.  Returns the bunch count.
+// Stage 2 (Eq. 2.2-2.5, Sec. 4.2.1): sub-step k of tile segment sg: angle and
+// mean bunch count at the sub-step midpoint, stochastic rounding with the
+// sub-step's own draw.  Returns the bunch count and the sub-step's record.
 template <bool SPH, bool FL, typename SM>
-__device__ __forceinline__ int substep(SM& S, int q, int sg, int k, long long base, const PropParams& pp,
+__device__ __forceinline__ int substep(const SM& S, float4& rec, int sg, int k, long long base, const PropParams& pp,
                                        const AtmParams& ap) {
     const float4 B = S.segB[sg];
     float dz_mid;
@@ -330,9 +330,7 @@ __device__ __forceinline__ int substep(SM& S, int q, int sg, int k, long long ba
     const float fl = floorf(nbar);
     const int N = (int)fl + (uk < nbar - fl ? 1 : 0);
     const float c2 = fmaxf(1.0f - sin2, 1e-30f), s2 = fmaxf(sin2, 1e-30f);
-    S.sub[q] = make_float4(c2 * rsqrtf(c2), sin2 > 0.0f ? s2 * rsqrtf(s2) : 0.0f, d,
-                           __int_as_float(sg | (k << kKShift)));
-    S.nsub_ph[q] = N;
+    rec = make_float4(c2 * rsqrtf(c2), sin2 > 0.0f ? s2 * rsqrtf(s2) : 0.0f, d, __int_as_float(sg | (k << kKShift)));
     return N;
 }
 
@@ -1276,8 +1274,10 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
 
     if constexpr (!SURR) {
         // ---- warps on their own: tiles of 32 segments, warp scans, no block barrier
-        WarpSmem& W = reinterpret_cast<WarpSmem*>(smem_raw)[t >> 5];
+        using WarpBuf = std::conditional_t<EX, WarpSmemPass, WarpSmem>;
+        WarpBuf& W = reinterpret_cast<WarpBuf*>(smem_raw)[t >> 5];
         const int lane = t & 31;
+        const unsigned int upto = 0xffffffffu >> (31 - lane), below = upto >> 1;   // lanes 0 .. lane, 0 .. lane - 1
         const long long n_wtiles = (pp.n + kWTile - 1) / kWTile;
         // `count` (at most 32) segments from `base` on; of their rounds of 32 bunches, those with
         // index part mod `parts` (a power of two); part 0 counts the segments and what they emit
@@ -1299,7 +1299,7 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
             // shower).  The draws stay keyed by the segments' own indices.
             int slot = lane;
             {
-                float key = 3.0e38f;   // empty slots last
+                unsigned int word = ~0u;   // empty slots last
                 if (Kt0 > 0) {
                     const float4 A = W.segA[lane], C = W.segC[lane];
                     float gx, gy;
@@ -1317,12 +1317,12 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                     }
                     gx -= pp.lv3_c[0];
                     gy -= pp.lv3_c[1];
-                    key = fmaf(gx, gx, gy * gy);
+                    word = __float_as_uint(fmaf(gx, gx, gy * gy));
                 }
                 // bitonic sort across the warp, ascending, of one 32-bit word per lane: the
                 // key's bits (a non-negative float orders as an unsigned integer) with its low
                 // five bits replaced by the slot, so that words are distinct and carry the slot
-                unsigned int word = (__float_as_uint(key) & ~31u) | (unsigned int)lane;
+                word = (word & ~31u) | (unsigned int)lane;
 #pragma unroll
                 for (int k = 2; k <= 32; k <<= 1) {
 #pragma unroll
@@ -1335,8 +1335,7 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                 }
                 slot = (int)(word & 31u);
             }
-            const int Kt = __shfl_sync(0xffffffffu, Kt0, slot);
-            W.perm[lane] = slot;
+            const int Kt = __shfl_sync(0xffffffffu, Kt0, slot);   // in that order from here on
             int incl = Kt;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -1344,61 +1343,62 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                 if (lane >= o) incl += y;
             }
             const int S_tot = __shfl_sync(0xffffffffu, incl, 31);
-            W.offK[lane] = incl - Kt;
-            if (lane == 31) W.offK[kWTile] = S_tot;
+            const int start = incl - Kt;   // the segment's first sub-step
             __syncwarp();
             for (int sub0 = 0; sub0 < S_tot; sub0 += kWSubCap) {
                 const int nsub = min(kWSubCap, S_tot - sub0);
-                // sub-step yields: a balanced run [q0, q1) per lane
-                const int per = (nsub + 31) >> 5;
-                const int q0 = min(lane * per, nsub), q1 = min(q0 + per, nsub);
-                int my_ph = 0;
+                // ---- sub-step yields, 32 at a time; those that emit are kept, with the index of
+                // their first bunch.  The segment of a lane's sub-step is the last one to start at or
+                // before it: the number of starts up to there, from one bit per start (a start is
+                // the first sub-step of exactly one segment; segments without sub-steps come last).
+                int J = 0, M = 0;   // sub-steps that emit, their bunches
                 unsigned int my_emit = 0;
-                if (q0 < q1) {
-                    int lo = 0, hi = kWTile;   // offK[lo] <= sub0 + q0 < offK[lo + 1]
-                    const int first = sub0 + q0;
-                    while (hi - lo > 1) {
-                        const int mid = (lo + hi) >> 1;
-                        if (W.offK[mid] <= first) lo = mid;
-                        else hi = mid;
-                    }
-                    int si = lo;
-                    for (int q = q0; q < q1; ++q) {
-                        const int qq = sub0 + q;
-                        while (W.offK[si + 1] <= qq) ++si;   // next non-empty segment
-                        const int sg = W.perm[si];
-                        const int N = substep<SPH, FL>(W, q, sg, qq - W.offK[si], base, pp, ap);
-                        my_ph += N;
+                for (int qb = 0; qb < nsub; qb += 32) {
+                    const int rel = start - (sub0 + qb);
+                    const int before = __popc(__ballot_sync(0xffffffffu, rel < 0 && Kt > 0));
+                    const unsigned int starts = __reduce_or_sync(0xffffffffu, Kt > 0 && (unsigned int)rel < 32u ? 1u << rel : 0u);
+                    const int si = (before + __popc(starts & upto) - 1) & 31;   // (a lane past nsub reads any)
+                    const int k = sub0 + qb + lane - __shfl_sync(0xffffffffu, start, si);
+                    const int sg = __shfl_sync(0xffffffffu, slot, si);
+                    int N = 0;
+                    float4 rec;
+                    if (qb + lane < nsub) {
+                        N = substep<SPH, FL>(W, rec, sg, k, base, pp, ap);
                         my_emit += (unsigned int)N * (unsigned int)W.bunch[sg];
                     }
+                    int ph = N;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int y = __shfl_up_sync(0xffffffffu, ph, o);
+                        if (lane >= o) ph += y;
+                    }
+                    const unsigned int emits = __ballot_sync(0xffffffffu, N > 0);
+                    if (N > 0) {
+                        const int j = J + __popc(emits & below);
+                        W.sub[j] = rec;
+                        W.first[j] = M + ph - N;
+                    }
+                    J += __popc(emits);
+                    M += __shfl_sync(0xffffffffu, ph, 31);
                 }
                 if (!TR || part == 0) emitted += my_emit;
-                int ph_incl = my_ph;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int y = __shfl_up_sync(0xffffffffu, ph_incl, o);
-                    if (lane >= o) ph_incl += y;
-                }
-                const int M = __shfl_sync(0xffffffffu, ph_incl, 31);
-                const int ph0 = ph_incl - my_ph;
+                W.first[J + lane] = 0x7fffffff;
                 __syncwarp();
-                // bunches over windows of the warp's bunch -> sub-step map
-                for (int p0 = 0; p0 < M; p0 += kWMapCap) {
-                    const int wn = min(kWMapCap, M - p0);
-                    int off = ph0;
-                    for (int q = q0; q < q1; ++q) {
-                        const int N = W.nsub_ph[q];
-                        const int a = max(off, p0), b = min(off + N, p0 + wn);
-                        for (int p = a; p < b; ++p) W.map[p - p0] = (unsigned int)q | ((unsigned int)(p - off) << kQBits);
-                        off += N;
-                    }
-                    __syncwarp();
+                // ---- bunches, 32 at a time.  A lane's sub-step is found like the segments above: at
+                // most 32 sub-steps begin in a round, the next ones after j_cur.  (A map entry per
+                // bunch, written by loops over the sub-steps, took 588 warp instructions per tile of
+                // 310 bunches, these look-ups about 130.)
+                int j_cur = -1, nq = 0;
+                for (int p0 = 0; p0 < M; p0 += 32) {
+                    const unsigned int rel = (unsigned int)(W.first[j_cur + 1 + lane] - p0);
+                    const unsigned int starts = __reduce_or_sync(0xffffffffu, rel < 32u ? 1u << rel : 0u);
+                    const int j = j_cur + __popc(starts & upto);
+                    j_cur += __popc(starts);
+                    const bool in = p0 + lane < M;
+                    const int ib = p0 + lane - W.first[j];
                     if constexpr (!EX) {
-                        const int skip = TR ? (part - (p0 >> 5)) & (parts - 1) : 0;   // rounds of other parts first
-                        for (int p = 32 * skip + lane; p < wn; p += TR ? 32 * parts : 32) {
-                            const unsigned int e = W.map[p];
-                            const int qs = (int)(e & ((1u << kQBits) - 1)), ib = (int)(e >> kQBits);
-                            const bool bey = bunch<false, SPH, REC, FL, TR, kModeMain, FIX>(W, qs, ib, true, base, pp, ap,
+                        if (in && (!TR || ((p0 >> 5) & (parts - 1)) == part)) {
+                            const bool bey = bunch<false, SPH, REC, FL, TR, kModeMain, FIX>(W, j, ib, true, base, pp, ap,
                                                                                            dp, op, sv, tcs, T);
                             // a bunch beyond the tables goes to the exact pass's queue (one
                             // reservation per group of converged lanes); when the queue is full its
@@ -1412,11 +1412,11 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                                     slot0 = pp.q_cap && __ldcg(scratch + 3) < pp.q_cap ? atomicAdd(scratch + 3, (unsigned int)__popc(m))
                                                                                        : 0xFFFFFFFFu;
                                 slot0 = __shfl_sync(m, slot0, leader);
-                                const unsigned int slot = slot0 + (unsigned int)__popc(m & ((1u << lane) - 1u));
-                                if (slot0 != 0xFFFFFFFFu && slot >= slot0 && slot < pp.q_cap) {
-                                    const int segk = __float_as_int(W.sub[qs].w);
+                                const unsigned int qslot = slot0 + (unsigned int)__popc(m & below);
+                                if (slot0 != 0xFFFFFFFFu && qslot >= slot0 && qslot < pp.q_cap) {
+                                    const int segk = __float_as_int(W.sub[j].w);
                                     const unsigned long long li = (unsigned long long)(base + (segk & ((1 << kKShift) - 1)));
-                                    reinterpret_cast<uint4*>(scratch + pp.q_off)[slot] =
+                                    reinterpret_cast<uint4*>(scratch + pp.q_off)[qslot] =
                                         make_uint4((uint32_t)li, (uint32_t)(li >> 32), (uint32_t)(segk >> kKShift), (uint32_t)ib);
                                 } else {
                                     any_beyond = true;
@@ -1424,42 +1424,31 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                             }
                         }
                     } else {
-                        // rounds of 32 bunches: those beyond the tables are queued (in the map
-                        // entries already read: a round's entries are never read again) and
-                        // propagated 32 at a time, so that the warp stays converged
-                        int nq = 0;
-                        for (int pw = 0;; pw += 32) {
-                            const bool last = pw + 32 >= wn;
-                            const int p = pw + lane;
-                            bool take = false;
-                            unsigned int e = 0;
-                            if (p < wn) {
-                                e = W.map[p];
-                                take = bunch<false, SPH, REC, FL, TR, kModeCheck>(W, (int)(e & ((1u << kQBits) - 1)),
-                                                                                 (int)(e >> kQBits), true, base, pp,
-                                                                                 ap, dp, op, sv, tcs, T);
+                        // bunches beyond the tables are queued and propagated 32 at a time, so that
+                        // the warp stays converged
+                        const bool last = p0 + 32 >= M;
+                        const bool take = in && bunch<false, SPH, REC, FL, TR, kModeCheck>(W, j, ib, true, base, pp, ap, dp,
+                                                                                          op, sv, tcs, T);
+                        const unsigned int m = __ballot_sync(0xffffffffu, take);
+                        if (take) {
+                            W.q_sub[nq + __popc(m & below)] = j;
+                            W.q_bunch[nq + __popc(m & below)] = ib;
+                        }
+                        nq += __popc(m);
+                        __syncwarp();
+                        while (nq >= 32 || (last && nq > 0)) {
+                            const int n_run = min(nq, 32);
+                            if (lane < n_run) {
+                                const int e = nq - n_run + lane;
+                                bunch<false, SPH, REC, FL, TR, kModeExact>(W, W.q_sub[e], W.q_bunch[e], true, base, pp, ap, dp,
+                                                                           op, sv, tcs, T);
                             }
-                            const unsigned int m = __ballot_sync(0xffffffffu, take);
+                            nq -= n_run;
                             __syncwarp();
-                            if (take) W.map[nq + __popc(m & ((1u << lane) - 1u))] = e;
-                            nq += __popc(m);
-                            __syncwarp();
-                            while (nq >= 32 || (last && nq > 0)) {
-                                const int n_run = min(nq, 32);
-                                if (lane < n_run) {
-                                    const unsigned int ex = W.map[nq - n_run + lane];
-                                    bunch<false, SPH, REC, FL, TR, kModeExact>(W, (int)(ex & ((1u << kQBits) - 1)),
-                                                                               (int)(ex >> kQBits), true, base, pp, ap,
-                                                                               dp, op, sv, tcs, T);
-                                }
-                                nq -= n_run;
-                                __syncwarp();
-                            }
-                            if (last) break;
                         }
                     }
-                    __syncwarp();
                 }
+                __syncwarp();
             }
             if constexpr (!EX) {   // the exact pass is to visit this tile
                 if (__any_sync(0xffffffffu, any_beyond) && lane == 0)
@@ -1501,7 +1490,7 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                     const long long base_l = li - lane;   // so that base + slot is the segment's index
                     if (act) {
                         import_segment<SPH, FL>(W, lane, pp.segs + li, pp, ap, dp, invalid, dropped, false);
-                        substep<SPH, FL>(W, lane, lane, (int)ent.z, base_l, pp, ap);
+                        substep<SPH, FL>(W, W.sub[lane], lane, (int)ent.z, base_l, pp, ap);
                         bunch<false, SPH, REC, FL, TR, kModeExact>(W, lane, (int)ent.w, true, base_l, pp, ap, dp, op, sv,
                                                                    tcs, T);
                     }
@@ -1552,7 +1541,8 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                     for (int q = q0; q < q1; ++q) {
                         const int qq = sub0 + q;
                         while (S.offK[sg + 1] <= qq) ++sg;   // next non-empty segment
-                        const int N = substep<SPH, FL>(S, q, sg, qq - S.offK[sg], base, pp, ap);
+                        const int N = substep<SPH, FL>(S, S.sub[q], sg, qq - S.offK[sg], base, pp, ap);
+                        S.nsub_ph[q] = N;
                         my_ph += N;
                         my_emit += (unsigned int)N * (unsigned int)S.bunch[sg];
                     }
@@ -1693,13 +1683,13 @@ cs_status launch_kernel(unsigned grid, cudaStream_t stream, const PropParams& pp
         CS_CUDA_TRY(cudaStreamIsCapturing(stream, &cap));
         auto pass = [&](auto kernel) {
             if (cap != cudaStreamCaptureStatusNone) {
-                kernel<<<grid_x, kThreads, kSmemExact, stream>>>(pp, ap, dp, op, ctr, sv);
+                kernel<<<grid_x, kThreads, kSmemPass, stream>>>(pp, ap, dp, op, ctr, sv);
                 return;
             }
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(grid_x);
             cfg.blockDim = dim3(kThreads);
-            cfg.dynamicSmemBytes = kSmemExact;
+            cfg.dynamicSmemBytes = kSmemPass;
             cfg.stream = stream;
             cudaLaunchAttribute at[1];
             at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1708,7 +1698,7 @@ cs_status launch_kernel(unsigned grid, cudaStream_t stream, const PropParams& pp
             cfg.numAttrs = 1;
             if (cudaLaunchKernelEx(&cfg, kernel, pp, ap, dp, op, ctr, sv) != cudaSuccess) {
                 cudaGetLastError();   // the attribute refused: an ordinary stream-ordered launch
-                kernel<<<grid_x, kThreads, kSmemExact, stream>>>(pp, ap, dp, op, ctr, sv);
+                kernel<<<grid_x, kThreads, kSmemPass, stream>>>(pp, ap, dp, op, ctr, sv);
             }
         };
         if (ap.spherical) {
@@ -1729,8 +1719,8 @@ cudaError_t set_exact_smem(int smem) {
     cudaError_t e = cudaFuncSetAttribute(propagate_kernel<false, S, 4, false, F, T>, attr, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<false, S, 4, true, F, T>, attr, smem);
     if (!T) {   // the exact pass of the table-tracer instances
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<false, S, 4, false, F, false, true>, attr, smem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<false, S, 4, true, F, false, true>, attr, smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<false, S, 4, false, F, false, true>, attr, (int)kSmemPass);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<false, S, 4, true, F, false, true>, attr, (int)kSmemPass);
     }
     if (!T && !F) {   // the fixed-configuration instances
         if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<false, S, 4, false, false, false, false, true>, attr, smem);
