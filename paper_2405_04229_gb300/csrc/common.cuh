@@ -14,6 +14,7 @@ constexpr double kPi = 3.14159265358979323846;
 constexpr double kLog2e = 1.4426950408889634;
 constexpr int kMaxLayers = 8;
 constexpr int kHashLevels = 3;   // telescope hash levels (zenith reach 45, 75, 82 deg)
+constexpr int kHashSubs = 3;     // lists of each level by arrival zenith (see TelHash)
 constexpr int kMaxNodes = 128;     // tabulated atmosphere
 constexpr double kTableRhoRef = 1.225e-3;   // [g/cm^3]: density = kTableRhoRef (n - 1) / kappa
 
@@ -77,6 +78,9 @@ struct AtmParams {
 // A uniform grid hash over the telescopes' reach discs for arrivals up to a
 // zenith: the grid origin and the cell size are whole metres, so cell corners
 // are exact in FP32; cell c lists the entries [cell_range[c].x, cell_range[c].y).
+// kHashSubs such tables follow one another, for arrivals whose sine squared is
+// at most sub_sin2[0], at most sub_sin2[1], and any up to sin2_max: less
+// steep arrivals reach fewer cells.
 struct TelHash {
     float gx0, gy0, cell, inv_cell;
     int gnx, gny;
@@ -84,7 +88,8 @@ struct TelHash {
     const int* cell_tel;      // telescope index of each entry (ascending within a cell)
     const float4* cell_data;  // planar: {x - corner_x, y - corner_y, z - h_obs, radius}; spherical: tel3
     float sin2_max;           // arrivals steeper than this need a wider hash or the full list
-    float bx0, bx1, by0, by1; // bounding box of all reach discs
+    float sub_sin2[kHashSubs - 1];
+    int n_cells;              // gnx * gny
 };
 
 struct DetParams {

@@ -12,9 +12,9 @@
 
 namespace {
 
-// the two hash levels serve arrivals up to 45 and 75 degrees zenith
-constexpr double kHashTheta[cs::kHashLevels] = {45.0 * 3.14159265358979323846 / 180.0, 75.0 * 3.14159265358979323846 / 180.0,
-                                                  82.0 * 3.14159265358979323846 / 180.0};
+// the largest arrival zeniths [deg] of the hash levels' lists; the last one is the level's own
+constexpr double kHashTheta[cs::kHashLevels][cs::kHashSubs] = {{24.0, 34.0, 45.0}, {60.0, 67.0, 75.0}, {77.0, 79.0, 82.0}};
+constexpr double kDeg = 3.14159265358979323846 / 180.0;
 
 void split(double v, float* hi, float* lo) {
     *hi = (float)v;
@@ -129,25 +129,33 @@ extern "C" cs_status cs_detector_create(const cs_detector_desc* d, cs_detector**
     std::vector<float4> cell_data[cs::kHashLevels];
     for (int level = 0; level < cs::kHashLevels && d->n_tel > 0; ++level) {
         cs::TelHash& H = p.hash[level];
-        const double theta_h = kHashTheta[level];
-        double reach_max = 0.0, x0 = 1e300, x1 = -1e300, y0 = 1e300, y1 = -1e300;
-        std::vector<double> reach(d->n_tel);
+        // ground points whose arrival line (zenith <= theta) passes within r of
+        // the centre lie within r / cos + |dz| tan of the centre's footprint
+        auto reach = [&](int i, double theta) {
+            const double* t = d->tel_xyzr + 4 * i;
+            return t[3] / cos(theta) + fabs(t[2] - d->h_obs) * tan(theta) + 0.01;
+        };
+        const double theta_h = kHashTheta[level][cs::kHashSubs - 1] * kDeg;
+        double reach_max = 0.0, reach_min = 0.0, x0 = 1e300, x1 = -1e300, y0 = 1e300, y1 = -1e300;
         for (int i = 0; i < d->n_tel; ++i) {
             const double* t = d->tel_xyzr + 4 * i;
-            // ground points whose arrival line (zenith <= theta_h) passes within r of
-            // the centre lie within r / cos + |dz| tan of the centre's footprint
-            reach[i] = t[3] / cos(theta_h) + fabs(t[2] - d->h_obs) * tan(theta_h) + 0.01;
-            reach_max = fmax(reach_max, reach[i]);
-            x0 = fmin(x0, t[0] - reach[i]); x1 = fmax(x1, t[0] + reach[i]);
-            y0 = fmin(y0, t[1] - reach[i]); y1 = fmax(y1, t[1] + reach[i]);
+            const double r = reach(i, theta_h);
+            reach_max = fmax(reach_max, r);
+            reach_min = fmax(reach_min, reach(i, kHashTheta[level][0] * kDeg));
+            x0 = fmin(x0, t[0] - r); x1 = fmax(x1, t[0] + r);
+            y0 = fmin(y0, t[1] - r); y1 = fmax(y1, t[1] + r);
         }
         // whole-metre origin and cell size: cell corners are exact in FP32.  Cells of half the
         // largest reach: a disc then covers ~25 cells, and a ground point's cell lists only the
         // spheres that can be near it (measured against 1, 1.5, 2 and 3 reaches: 2 % faster on
-        // the 100-telescope grid and 4 % on the 2,000 inclined-shower telescopes than 2 reaches)
+        // the 100-telescope grid and 4 % on the 2,000 inclined-shower telescopes than 2 reaches).
+        // On the sphere, whose entries do not depend on the cells, of half the first list's reach
+        // as long as the discs' cells stay few enough.
         x0 = floor(x0);
         y0 = floor(y0);
         double cell = fmax(ceil(0.5 * reach_max), 1.0);
+        const double first = fmax(ceil(0.5 * reach_min), 1.0);
+        if (p.spherical && (double)d->n_tel * (2.0 * reach_max / first + 1.0) * (2.0 * reach_max / first + 1.0) < 4e6) cell = first;
         if (fabs(x0) > 8e6 || fabs(y0) > 8e6 || fabs(x1) > 8e6 || fabs(y1) > 8e6) {
             delete h;
             return CS_ERR_INVALID_ARG;
@@ -156,27 +164,53 @@ extern "C" cs_status cs_detector_create(const cs_detector_desc* d, cs_detector**
         while ((double)gnx * gny > 4e6) { cell *= 2.0; gnx = (int)ceil((x1 - x0) / cell); gny = (int)ceil((y1 - y0) / cell); }
         gnx = gnx < 1 ? 1 : gnx;
         gny = gny < 1 ? 1 : gny;
-        std::vector<std::vector<int>> lists((size_t)gnx * gny);
-        for (int i = 0; i < d->n_tel; ++i) {   // ascending index within every cell
+        const size_t n_cells = (size_t)gnx * gny;
+        // the kernel's cell index comes from FP32 coordinates: a few ulps at the grid's far corner
+        const double slack = 4e-7 * fmax(fmax(fabs(x0), fabs(x1)), fmax(fabs(y0), fabs(y1)));
+        // calls f(row, first column, last column) for the cells that the disc of radius r about
+        // telescope i touches
+        auto for_rows = [&](int i, double r, auto&& f) {
             const double* t = d->tel_xyzr + 4 * i;
-            int cx0 = (int)floor((t[0] - reach[i] - x0) / cell), cx1 = (int)floor((t[0] + reach[i] - x0) / cell);
-            int cy0 = (int)floor((t[1] - reach[i] - y0) / cell), cy1 = (int)floor((t[1] + reach[i] - y0) / cell);
-            for (int cy = cy0 < 0 ? 0 : cy0; cy <= cy1 && cy < gny; ++cy)
-                for (int cx = cx0 < 0 ? 0 : cx0; cx <= cx1 && cx < gnx; ++cx)
-                    lists[(size_t)cy * gnx + cx].push_back(i);
-        }
-        range[level].resize(lists.size());
-        for (size_t c = 0; c < lists.size(); ++c) {
-            const double cx0 = x0 + (double)(c % gnx) * cell, cy0 = y0 + (double)(c / gnx) * cell;
-            range[level][c].x = (int)cell_tel[level].size();
-            for (int i : lists[c]) {
-                const double* t = d->tel_xyzr + 4 * i;
-                cell_tel[level].push_back(i);
-                cell_data[level].push_back(p.spherical ? tel3[i]
-                                                       : make_float4((float)(t[0] - cx0), (float)(t[1] - cy0),
-                                                                     (float)(t[2] - d->h_obs), (float)t[3]));
+            const int r0 = std::max((int)floor((t[1] - r - y0) / cell), 0), r1 = std::min((int)floor((t[1] + r - y0) / cell), gny - 1);
+            for (int row = r0; row <= r1; ++row) {
+                const double dy = fmax(fmax(y0 + row * cell - t[1], t[1] - (y0 + (row + 1) * cell)), 0.0);
+                const double half = sqrt(fmax(r * r - dy * dy, 0.0));
+                const int c0 = std::max((int)floor((t[0] - half - x0) / cell), 0);
+                const int c1 = std::min((int)floor((t[0] + half - x0) / cell), gnx - 1);
+                if (c0 <= c1) f(row, c0, c1);
             }
-            range[level][c].y = (int)cell_tel[level].size();
+        };
+        range[level].resize(n_cells * cs::kHashSubs);
+        std::vector<int> fill(n_cells);
+        for (int sub = 0; sub < cs::kHashSubs; ++sub) {
+            int2* er = range[level].data() + sub * n_cells;
+            std::fill(fill.begin(), fill.end(), 0);
+            for (int i = 0; i < d->n_tel; ++i) {
+                for_rows(i, reach(i, kHashTheta[level][sub] * kDeg) + slack, [&](int row, int c0, int c1) {
+                    for (int c = c0; c <= c1; ++c) ++fill[(size_t)row * gnx + c];
+                });
+            }
+            int at = (int)cell_tel[level].size();
+            for (size_t c = 0; c < n_cells; ++c) {
+                er[c] = make_int2(at, at + fill[c]);
+                at += fill[c];
+                fill[c] = er[c].x;
+            }
+            cell_tel[level].resize(at);
+            cell_data[level].resize(at);
+            for (int i = 0; i < d->n_tel; ++i) {   // ascending index within every cell
+                const double* t = d->tel_xyzr + 4 * i;
+                for_rows(i, reach(i, kHashTheta[level][sub] * kDeg) + slack, [&](int row, int c0, int c1) {
+                    for (int c = c0; c <= c1; ++c) {
+                        const int e = fill[(size_t)row * gnx + c]++;
+                        cell_tel[level][e] = i;
+                        cell_data[level][e] = p.spherical ? tel3[i]
+                                                          : make_float4((float)(t[0] - (x0 + (double)c * cell)),
+                                                                        (float)(t[1] - (y0 + (double)row * cell)),
+                                                                        (float)(t[2] - d->h_obs), (float)t[3]);
+                    }
+                });
+            }
         }
         H.gx0 = (float)x0;
         H.gy0 = (float)y0;
@@ -184,17 +218,19 @@ extern "C" cs_status cs_detector_create(const cs_detector_desc* d, cs_detector**
         H.inv_cell = (float)(1.0 / cell);
         H.gnx = gnx;
         H.gny = gny;
-        H.bx0 = (float)x0; H.bx1 = (float)(x0 + gnx * cell);
-        H.by0 = (float)y0; H.by1 = (float)(y0 + gny * cell);
+        H.n_cells = (int)n_cells;
         // on the sphere the local vertical at a ground point in the box leans from
         // the frame's z axis by up to the box's extent / r_g: photons steeper than
-        // the hash's zenith in the local frame must be steeper in the frame's too
-        double theta = theta_h;
+        // a list's zenith in the local frame must be steeper in the frame's too
+        double lean = 0.0;
         if (p.spherical) {
             const double ex = fmax(fabs(x0), fabs(x0 + gnx * cell)), ey = fmax(fabs(y0), fabs(y0 + gny * cell));
-            theta -= 1.01 * sqrt(ex * ex + ey * ey) / (p.R + d->h_obs) + 1e-6;
+            lean = 1.01 * sqrt(ex * ex + ey * ey) / (p.R + d->h_obs) + 1e-6;
         }
-        H.sin2_max = (float)(sin(theta) * sin(theta));
+        for (int sub = 0; sub < cs::kHashSubs; ++sub) {
+            const double theta = fmax(kHashTheta[level][sub] * kDeg - lean, 0.0);
+            (sub + 1 < cs::kHashSubs ? H.sub_sin2[sub] : H.sin2_max) = (float)(sin(theta) * sin(theta));
+        }
     }
     const size_t o_tel = 0;
     const size_t o_lo = align_up(o_tel + tel.size() * sizeof(float4));

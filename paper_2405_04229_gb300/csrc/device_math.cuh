@@ -124,6 +124,13 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return y;
 }
 
+// of a normal number: the same value as rsqrtf without its care for subnormal arguments
+__device__ __forceinline__ float rsqrt_approx(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // sin and cos of 2 pi u for u in [0, 1): exact quadrant reduction of 4u and
 // Taylor polynomials on |x| <= pi/4 (truncation below 3e-8).
 __device__ __forceinline__ void sincos_2pi(float u, float& s, float& c) {
@@ -153,12 +160,14 @@ __device__ __forceinline__ float delta_at(const AtmParams& a, float dz) {
         // operands, no indexed parameter loads)
         float D = a.lay_D[0], c2 = a.lay_c2[0];
 #pragma unroll
-        for (int k = 1; k < kMaxLayers; ++k)
-            if (k < a.n_layers && dz >= a.lay_lo[k]) {
+        for (int k = 1; k < kMaxLayers; ++k) {
+            if (k >= a.n_layers) break;
+            if (dz >= a.lay_lo[k]) {
                 D = a.lay_D[k];
                 c2 = a.lay_c2[k];
             }
-        return D * exp2f(c2 * dz);
+        }
+        return D * ex2_approx(c2 * dz);
     }
     if (a.kind == CS_ATM_LINEAR) return dz >= a.lin_top_rel ? a.lin_d1 : a.lin_d0 + a.lin_slope * dz;
     if (a.kind == CS_ATM_TABLE) {
@@ -169,7 +178,7 @@ __device__ __forceinline__ float delta_at(const AtmParams& a, float dz) {
             if (__ldg(a.node_lo + mid) <= dz) lo = mid;
             else hi = mid;
         }
-        return __ldg(a.node_d + lo) * exp2f(__ldg(a.node_c2 + lo) * (dz - __ldg(a.node_lo + lo)));
+        return __ldg(a.node_d + lo) * ex2_approx(__ldg(a.node_c2 + lo) * (dz - __ldg(a.node_lo + lo)));
     }
     return a.hom_delta;
 }

@@ -45,7 +45,7 @@ struct TileSmem {
     float4 segC[kTile];   // ground intercept G, float-float x and y | start point (hi), radial P component
     float4 segD[kTile];   // G in histogram cells, float-float x and y | start point (lo), 1 / r
     double t0[kTile];
-    float g[kTile], z2[kTile];
+    float g[kTile], z2[kTile], inv_b[kTile];   // 1 / gamma^2, z^2 x yield constant, 1 / bunch
     int shower[kTile];
     int bunch[kTile];     // photons per bunch of the segment's shower
     int offK[kTile + 1];
@@ -66,7 +66,7 @@ constexpr int kWSubCap = 128;           // sub-steps per warp round
 struct WarpSmem {
     float4 segA[kWTile], segB[kWTile], segC[kWTile], segD[kWTile];   // as in TileSmem
     double t0[kWTile];
-    float g[kWTile], z2[kWTile];
+    float g[kWTile], z2[kWTile], inv_b[kWTile];
     int shower[kWTile];
     int bunch[kWTile];
     float4 sub[kWSubCap];        // the round's sub-steps that emit a bunch, in order
@@ -209,7 +209,7 @@ __device__ __forceinline__ int import_segment(SM& S, int t, const cs_segment* se
         invalid += 1;
         return 0;
     }
-    const float inv_n = rsqrtf(n2);
+    const float inv_n = rsqrt_approx(n2);
     const float Px = dir.x * inv_n, Py = dir.y * inv_n, Pz = dir.z * inv_n;
     const float L = dir.w;
     const int K = substep_count(L, pp.s_max, pp.s_max_lo);
@@ -241,14 +241,16 @@ __device__ __forceinline__ int import_segment(SM& S, int t, const cs_segment* se
         const float dvx = x_hi * inv_r, dvy = y_hi * inv_r, dvz = -lift * inv_r;   // v - z-hat
         const float Pr = Px * dvx + Py * dvy + Pz * (1.0f + dvz);
         S.segA[t] = make_float4(Px, Py, Pz, 1.0f / (1.0f - Pz));
-        S.segB[t] = make_float4(Hs, dvz, L / (float)K, rsqrtf(1.0f - g) * kInvC);
+        S.segB[t] = make_float4(Hs, dvz, L / (float)K, rsqrt_approx(1.0f - g) * kInvC);
         S.segC[t] = make_float4(x_hi, y_hi, z_hi, Pr);
         S.segD[t] = make_float4(x_lo, y_lo, z_lo, inv_r);
         S.t0[t] = zt.y;
         S.g[t] = g;
-        S.z2[t] = z * z;
+        S.z2[t] = (FL ? pp.fl_yd : ap.ft) * (z * z);
         S.shower[t] = (int)shower;
-        S.bunch[t] = pp.shower_bunch ? __ldg(pp.shower_bunch + shower) : pp.bunch;
+        const int bsz = pp.shower_bunch ? __ldg(pp.shower_bunch + shower) : pp.bunch;
+        S.bunch[t] = bsz;
+        S.inv_b[t] = rcp_approx((float)bsz);
         return K;
     }
     if (filter && pp.lv1 && lv1_drop<false>(pp, dp, x_hi, x_lo, y_hi, y_lo, z_hi, z_lo, Hs_hi + Hs_lo, Px, Py, Pz)) {
@@ -271,7 +273,7 @@ __device__ __forceinline__ int import_segment(SM& S, int t, const cs_segment* se
         two_sum(s, e + (y_lo - py_l), Gyh, Gyl);
     }
     S.segA[t] = make_float4(Px, Py, Pz, 1.0f / (1.0f - Pz));
-    S.segB[t] = make_float4(Hs_hi, Hs_lo, L / (float)K, rsqrtf(1.0f - g) * kInvC);
+    S.segB[t] = make_float4(Hs_hi, Hs_lo, L / (float)K, rsqrt_approx(1.0f - g) * kInvC);
     S.segC[t] = make_float4(Gxh, Gxl, Gyh, Gyl);
     if (dp.nx > 0) {
         float s, e, cxh, cxl, cyh, cyl;
@@ -283,9 +285,11 @@ __device__ __forceinline__ int import_segment(SM& S, int t, const cs_segment* se
     }
     S.t0[t] = zt.y;
     S.g[t] = g;
-    S.z2[t] = z * z;
+    S.z2[t] = (FL ? pp.fl_yd : ap.ft) * (z * z);
     S.shower[t] = (int)shower;
-    S.bunch[t] = pp.shower_bunch ? __ldg(pp.shower_bunch + shower) : pp.bunch;
+    const int bsz = pp.shower_bunch ? __ldg(pp.shower_bunch + shower) : pp.bunch;
+        S.bunch[t] = bsz;
+        S.inv_b[t] = rcp_approx((float)bsz);
     return K;
 }
 
@@ -322,15 +326,15 @@ __device__ __forceinline__ int substep(const SM& S, float4& rec, int sg, int k, 
     // 1 - 1/(beta n)^2 without forming 1/(beta n)^2 (cancellation-free)
     const float sin2 = (d * (2.0f + d) - onepd * onepd * g) * rcp_approx(onepd * onepd * (1.0f - g));
     float nbar = 0.0f;
-    if constexpr (FL) nbar = pp.fl_yd * S.z2[sg] * d * B.z * rcp_approx((float)S.bunch[sg]);   // Eq. 2.6
-    else if (sin2 > 0.0f) nbar = ap.ft * S.z2[sg] * sin2 * B.z * rcp_approx((float)S.bunch[sg]);
+    if constexpr (FL) nbar = S.z2[sg] * d * B.z * S.inv_b[sg];   // Eq. 2.6
+    else if (sin2 > 0.0f) nbar = S.z2[sg] * sin2 * B.z * S.inv_b[sg];
     const unsigned long long gid = pp.seg_base + (unsigned long long)(base + sg);
     const uint4 rc = philox_rk((uint32_t)gid, (uint32_t)(gid >> 32), (uint32_t)k, 0xFFFFFFFFu, pp.rk);
     const float uk = uniform24(rc.x);
     const float fl = floorf(nbar);
     const int N = (int)fl + (uk < nbar - fl ? 1 : 0);
     const float c2 = fmaxf(1.0f - sin2, 1e-30f), s2 = fmaxf(sin2, 1e-30f);
-    rec = make_float4(c2 * rsqrtf(c2), sin2 > 0.0f ? s2 * rsqrtf(s2) : 0.0f, d, __int_as_float(sg | (k << kKShift)));
+    rec = make_float4(c2 * rsqrt_approx(c2), sin2 > 0.0f ? s2 * rsqrt_approx(s2) : 0.0f, d, __int_as_float(sg | (k << kKShift)));
     return N;
 }
 
@@ -348,13 +352,13 @@ __device__ __forceinline__ void hist_add(const OutParams& op, unsigned int key, 
 
 // Telescopes: the sphere whose centre is closest to the arrival line, if
 // closer than its radius (ties: lowest index).  Arrivals within the hash's
-// zenith range (`hashed`; the caller has checked the box of all reach discs)
-// test the entries of their grid cell: cell_delta(entry, corner_x, corner_y,
-// ddx, ddy, ddz) gives the centre minus the ground point.  Steeper arrivals
-// test every sphere through full_delta(index, ddx, ddy, ddz, radius).
+// zenith range (`hashed`) test the entries of their grid cell in the list for
+// their own sine squared s2: cell_delta(entry, corner_x, corner_y, ddx, ddy,
+// ddz) gives the centre minus the ground point.  Steeper arrivals test every
+// sphere through full_delta(index, ddx, ddy, ddz, radius).
 template <typename CellDelta, typename FullDelta>
-__device__ __forceinline__ int hit_telescope(const DetParams& dp, const TelHash& H, bool hashed, float x, float y, float ugx,
-                                             float ugy, float ugz, CellDelta cell_delta, FullDelta full_delta) {
+__device__ __forceinline__ int hit_telescope(const DetParams& dp, const TelHash& H, bool hashed, float s2, float x, float y,
+                                             float ugx, float ugy, float ugz, CellDelta cell_delta, FullDelta full_delta) {
     int best = -1;
     float best_d2 = 3.0e38f;
     auto test = [&](float ddx, float ddy, float ddz, float r, int id) {
@@ -368,8 +372,9 @@ __device__ __forceinline__ int hit_telescope(const DetParams& dp, const TelHash&
     if (hashed) {
         const int cx = (int)((x - H.gx0) * H.inv_cell);
         const int cy = (int)((y - H.gy0) * H.inv_cell);
-        if (cx < 0 || cx >= H.gnx || cy < 0 || cy >= H.gny) return -1;
-        const int2 er = __ldg(H.cell_range + (cy * H.gnx + cx));
+        // (a point less than a cell outside the grid lands in its edge cell: beyond every reach, it hits nothing)
+        if ((unsigned int)cx >= (unsigned int)H.gnx || (unsigned int)cy >= (unsigned int)H.gny) return -1;
+        const int2 er = __ldg(H.cell_range + (cy * H.gnx + cx + (s2 > H.sub_sin2[0] ? H.n_cells : 0) + (s2 > H.sub_sin2[1] ? H.n_cells : 0)));
         if (er.x == er.y) return -1;   // no reach disc covers this cell
         const float cx0 = fmaf((float)cx, H.cell, H.gx0), cy0 = fmaf((float)cy, H.cell, H.gy0);   // exact
         for (int e = er.x; e < er.y; ++e) {
@@ -868,6 +873,7 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
             // the path never meets the observation level: missed
         } else if (c_trans && !(u3 < Tr)) {
             status = CS_ST_ABSORBED;
+            T.absorbed += b;
         } else {
             const int sh = S.shower[sg];
             if (c_hist) {   // ground cell = floor(G_cells + r / d); rounding < 3e-5 cells
@@ -876,6 +882,7 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                 const int iy = (int)floorf(D.z + fmaf(ry, dp.inv_dy, D.w));
                 if (ix >= 0 && ix < dp.nx && iy >= 0 && iy < dp.ny) {
                     bin = iy * dp.nx + ix;
+                    T.hist += b;
                     hist_add(op, (unsigned int)(sh * dp.ny * dp.nx + bin), b);
                 }
             }
@@ -887,14 +894,14 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                 // first, its fields are constant operands (no indexed parameter loads)
                 const bool lvl0 = s2 <= dp.hash[0].sin2_max;
                 auto detect = [&](const TelHash& H, const bool hashed) {
-                if (!hashed || (x >= H.bx0 && x < H.bx1 && y >= H.by0 && y < H.by1)) {
+                {
                     float ugz = uz;
                     if (c_refr) {
                         const float c2 = fmaxf(1.0f - s2, 1e-30f);
-                        ugz = -c2 * rsqrtf(c2);
+                        ugz = -c2 * rsqrt_approx(c2);
                     }
                     tel = hit_telescope(
-                        dp, H, hashed, x, y, ux * sc, uy * sc, ugz,
+                        dp, H, hashed, s2, x, y, ux * sc, uy * sc, ugz,
                         [&](const float4& D, float cx0, float cy0, float& ddx, float& ddy, float& ddz) {
                             ddx = D.x - ((Cg.x - cx0) + (Cg.y + rx));
                             ddy = D.y - ((Cg.z - cy0) + (Cg.w + ry));
@@ -920,6 +927,7 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                 if (__all_sync(__activemask(), lvl0)) detect(dp.hash[0], true);
                 else detect(dp.hash[lvl0 ? 0 : (s2 <= dp.hash[1].sin2_max ? 1 : 2)], s2 <= dp.hash[2].sin2_max);
                 if (tel >= 0) {
+                    T.tel += b;
                     const size_t slot = (size_t)sh * dp.n_tel + tel;
                     atomicAdd(op.tel_counts + slot, (unsigned long long)b);
                     if (c_time) atomicAdd(op.tel_time + slot, (double)b * (S.t0[sg] + (double)t_rel));
@@ -973,6 +981,7 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
             // turned above the ground: missed
         } else if (c_trans && !(u3 < Tr)) {
             status = CS_ST_ABSORBED;
+            T.absorbed += b;
         } else {
             const int sh = S.shower[sg];
             if (c_hist) {
@@ -980,6 +989,7 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                 const int iy = (int)floorf(((y - dp.hy0_hi) + (yl - dp.hy0_lo)) * dp.inv_dy);
                 if (ix >= 0 && ix < dp.nx && iy >= 0 && iy < dp.ny) {
                     bin = iy * dp.nx + ix;
+                    T.hist += b;
                     hist_add(op, (unsigned int)(sh * dp.ny * dp.nx + bin), b);
                 }
             }
@@ -993,9 +1003,9 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                 const float sg2 = ugx * ugx + ugy * ugy;
                 const bool lvl0 = sg2 <= dp.hash[0].sin2_max;
                 auto detect = [&](const TelHash& H, const bool hashed) {
-                if (!hashed || (xs >= H.bx0 && xs < H.bx1 && ys >= H.by0 && ys < H.by1)) {
+                {
                     tel = hit_telescope(
-                        dp, H, hashed, xs, ys, ugx, ugy, ugz,
+                        dp, H, hashed, sg2, xs, ys, ugx, ugy, ugz,
                         [&](const float4& D, float cx0, float cy0, float& ddx, float& ddy, float& ddz) {
                             ddx = D.x - ((x - cx0) + xl);
                             ddy = D.y - ((y - cy0) + yl);
@@ -1020,6 +1030,7 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                 if (__all_sync(__activemask(), lvl0)) detect(dp.hash[0], true);
                 else detect(dp.hash[lvl0 ? 0 : (sg2 <= dp.hash[1].sin2_max ? 1 : 2)], sg2 <= dp.hash[2].sin2_max);
                 if (tel >= 0) {
+                    T.tel += b;
                     const size_t slot = (size_t)sh * dp.n_tel + tel;
                     atomicAdd(op.tel_counts + slot, (unsigned long long)b);
                     if (c_time) atomicAdd(op.tel_time + slot, (double)b * (S.t0[sg] + (double)t_rel));
@@ -1110,7 +1121,7 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
             const float gvx = Gx * irg, gvy = Gy * irg, gvz = (Gz - h_obs_f) * irg;   // v_G - z-hat
             const float uvG = ux * gvx + uy * gvy + uz * (1.0f + gvz);
             float tx = ux - uvG * gvx, ty = uy - uvG * gvy, tz = uz - uvG * (1.0f + gvz);
-            const float tn = rsqrtf(fmaxf(tx * tx + ty * ty + tz * tz, 1e-30f));
+            const float tn = rsqrt_approx(fmaxf(tx * tx + ty * ty + tz * tz, 1e-30f));
             tx *= tn;
             ty *= tn;
             tz *= tn;
@@ -1139,6 +1150,7 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
             const float xs = x + xl, ys = y + yl;   // single floats for the box and hash tests
             if (c_trans && !(u3 < Tr)) {
                 status = CS_ST_ABSORBED;
+                T.absorbed += b;
             } else {
                 const int sh = S.shower[sg];
                 if (c_hist) {
@@ -1146,6 +1158,7 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                     const int iy = (int)floorf(((y - dp.hy0_hi) + (yl - dp.hy0_lo)) * dp.inv_dy);
                     if (ix >= 0 && ix < dp.nx && iy >= 0 && iy < dp.ny) {
                         bin = iy * dp.nx + ix;
+                        T.hist += b;
                         hist_add(op, (unsigned int)(sh * dp.ny * dp.nx + bin), b);
                     }
                 }
@@ -1159,16 +1172,21 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                         ugz = -cos_g * (1.0f + gvz) + sin_g * tz;
                     }
                     const float sg2 = ugx * ugx + ugy * ugy;
-                    const bool lvl0 = sg2 <= dp.hash[0].sin2_max;
-                    auto detect = [&](const TelHash& H, const bool hashed) {
-                    if (!hashed || (xs >= H.bx0 && xs < H.bx1 && ys >= H.by0 && ys < H.by1)) {
+                    // the narrowest hash that serves every active lane (the entries are in frame
+                    // coordinates, so any that serves gives the same hit): one copy of the search
+                    const int lvl = __all_sync(__activemask(), sg2 <= dp.hash[0].sin2_max)   ? 0
+                                    : __all_sync(__activemask(), sg2 <= dp.hash[1].sin2_max) ? 1
+                                                                                             : 2;
+                    const TelHash& H = dp.hash[lvl];
+                    const bool hashed = sg2 <= H.sin2_max;
+                    {
                         auto delta3 = [&](const float4& T3, float& ddx, float& ddy, float& ddz) {
                             ddx = (T3.x - Gx) - Gxl;
                             ddy = (T3.y - Gy) - Gyl;
                             ddz = (T3.z - Gz) - Gzl;
                         };
                         tel = hit_telescope(
-                            dp, H, hashed, xs, ys, ugx, ugy, ugz,
+                            dp, H, hashed, sg2, xs, ys, ugx, ugy, ugz,
                             [&](const float4& D, float, float, float& ddx, float& ddy, float& ddz) { delta3(D, ddx, ddy, ddz); },
                             [&](int it, float& ddx, float& ddy, float& ddz, float& r) {
                                 const float4 T3 = __ldg(dp.tel3 + it);
@@ -1181,10 +1199,8 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                             pix = optics_survival(dp, pp, gid, k, i, inv_l, pix);
                         }
                     }
-                    };
-                    if (__all_sync(__activemask(), lvl0)) detect(dp.hash[0], true);
-                    else detect(dp.hash[lvl0 ? 0 : (sg2 <= dp.hash[1].sin2_max ? 1 : 2)], sg2 <= dp.hash[2].sin2_max);
                     if (tel >= 0) {
+                        T.tel += b;
                         const size_t slot = (size_t)sh * dp.n_tel + tel;
                         atomicAdd(op.tel_counts + slot, (unsigned long long)b);
                         if (c_time) atomicAdd(op.tel_time + slot, (double)b * (S.t0[sg] + (double)t_rel));
@@ -1194,10 +1210,7 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
             }
         }
     }
-    T.absorbed += status == CS_ST_ABSORBED ? b : 0;
     T.upward += status == CS_ST_UPWARD ? b : 0;
-    T.hist += bin >= 0 ? b : 0;
-    T.tel += tel >= 0 ? b : 0;
     if (REC) emit_record(op, gid, k, i, x, xl, y, yl, t_rel, inv_l, tel, bin, status, pix);
     return false;
 }
