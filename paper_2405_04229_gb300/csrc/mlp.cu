@@ -16,7 +16,7 @@
 #include <chrono>
 #include <vector>
 
-#include "mlp_tc.cuh"
+#include "mlp_step.cuh"
 
 struct cs_surrogate {
     float* d_p = nullptr;             // FP32 master parameters
@@ -350,14 +350,7 @@ __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, 
                             const unsigned int* __restrict__ step_ctr) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= kNParams) return;
-    const float4 sc = sched[*step_ctr];
-    const float lr = sc.x, c1 = sc.y, c2 = sc.z;
-    if ((i >= kOffW4 + kNOut * kHid && i < kOffB4) || i >= kOffB4 + kNOut) return;   // padding
-    const float gi = g[i];
-    const float mi = 0.9f * m[i] + 0.1f * gi, vi = 0.999f * v[i] + 0.001f * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
+    adam_update(i, g[i], p, m, v, sched[*step_ctr]);
 }
 
 // BF16 copies of W2, W3, W4 (same [n][k] layout as the masters).
@@ -653,16 +646,18 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
     float* T = (float*)A(n_all * 3 * sizeof(float));
     float* Xb = (float*)A((size_t)B * 3 * sizeof(float));
     float* Tb = (float*)A((size_t)B * 3 * sizeof(float));
+    const bool fused = step_fused(B);   // the step in two kernels; other batch sizes pass through global memory
+    const size_t Bu = fused ? 1 : (size_t)B;
     Work w;
-    w.H1 = (float*)A((size_t)B * kHid * 4);
-    w.H2 = (float*)A((size_t)B * kHid * 4);
-    w.H3 = (float*)A((size_t)B * kHid * 4);
-    w.dH = (float*)A((size_t)B * kHid * 4);
-    w.dZ = (float*)A((size_t)B * kHid * 4);
-    w.Y = (float*)A((size_t)B * kNOutP * 4);
-    w.dY = (float*)A((size_t)B * kNOutP * 4);
+    w.H1 = (float*)A(Bu * kHid * 4);
+    w.H2 = (float*)A(Bu * kHid * 4);
+    w.H3 = (float*)A(Bu * kHid * 4);
+    w.dH = (float*)A(Bu * kHid * 4);
+    w.dZ = (float*)A(Bu * kHid * 4);
+    w.Y = (float*)A(Bu * kNOutP * 4);
+    w.dY = (float*)A(Bu * kNOutP * 4);
     w.loss = (float*)A(256);
-    w.part = (float*)A(work_part_floats(B) * 4);
+    w.part = (float*)A((fused ? step_part_floats(B) : work_part_floats(B)) * 4);
     float* p = (float*)A(kNParams * 4);
     float* pr = (float*)A(kNParams * 4);
     float* g = (float*)A(kNParams * 4);
@@ -806,11 +801,12 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
             hs[step - 1] = make_float4((float)lr, (float)(1.0 - pow(0.9, step)), (float)(1.0 - pow(0.999, step)), 0.0f);
         }
         float4* sched = (float4*)A(hs.size() * sizeof(float4));
-        unsigned int* step_ctr = (unsigned int*)A(sizeof(unsigned int));
+        unsigned int* step_ctr = (unsigned int*)A(2 * sizeof(unsigned int));   // and the fused reduction's own
         if (!sched || !step_ctr) { cudaFree(d_base); cleanup(); return CS_ERR_CUDA; }
         cudaMemcpy(sched, hs.data(), hs.size() * sizeof(float4), cudaMemcpyHostToDevice);
-        cudaMemset(step_ctr, 0, sizeof(unsigned int));
-        if ((e = cudaDeviceSynchronize()) != cudaSuccess) {
+        cudaMemset(step_ctr, 0, 2 * sizeof(unsigned int));
+        if (fused) e = step_attributes();
+        if (e != cudaSuccess || (e = cudaDeviceSynchronize()) != cudaSuccess) {
             set_last_error("surrogate training set-up", e);
             cudaFree(d_base);
             cleanup();
@@ -819,7 +815,25 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
         cudaStream_t ts = nullptr;
         cudaGraph_t graphs[2] = {nullptr, nullptr};
         cudaGraphExec_t execs[2] = {nullptr, nullptr};
+        StepArgs sa = {};
+        ReduceArgs ra = {};
+        if (fused) {
+            step_layout(w.part, B, sa, ra);
+            sa.X = X; sa.T = T; sa.Wt = Wt;
+            sa.n = nt;
+            sa.key0 = k0; sa.key1 = k1;
+            sa.step = ra.step = step_ctr;
+            sa.step_red = ra.step_red = step_ctr + 1;
+            sa.p = ra.p = p;
+            ra.m = m; ra.v = v;
+            ra.sched = sched;
+            ra.loss_out = w.loss;
+        }
         auto enqueue_step = [&]() {
+            if (fused) {
+                step_launch(sa, ra, ts);
+                return;
+            }
             gather_kernel<<<(B + 255) / 256, 256, 0, ts>>>(X, T, Wt, nt, B, k0, k1, step_ctr, Xb, Tb, Wb);
             round_weights_kernel<<<(kNParams + 255) / 256, 256, 0, ts>>>(p, pr);
             cudaMemsetAsync(g, 0, kNParams * 4, ts);
@@ -1014,15 +1028,17 @@ extern "C" cs_status cs_mlp_loss_grad(const float* params, const float* x, const
     Work w;
     float *X = A((size_t)B * 12), *T = A((size_t)B * 12), *p = A(kNParams * 4), *pr = A(kNParams * 4),
           *g = A(kNParams * 4);
-    w.H1 = A((size_t)B * kHid * 4);
-    w.H2 = A((size_t)B * kHid * 4);
-    w.H3 = A((size_t)B * kHid * 4);
-    w.dH = A((size_t)B * kHid * 4);
-    w.dZ = A((size_t)B * kHid * 4);
-    w.Y = A((size_t)B * kNOutP * 4);
-    w.dY = A((size_t)B * kNOutP * 4);
+    const bool fused = step_fused(B);
+    const size_t Bu = fused ? 1 : (size_t)B;
+    w.H1 = A(Bu * kHid * 4);
+    w.H2 = A(Bu * kHid * 4);
+    w.H3 = A(Bu * kHid * 4);
+    w.dH = A(Bu * kHid * 4);
+    w.dZ = A(Bu * kHid * 4);
+    w.Y = A(Bu * kNOutP * 4);
+    w.dY = A(Bu * kNOutP * 4);
     w.loss = A(256);
-    w.part = A(work_part_floats(B) * 4);
+    w.part = A((fused ? step_part_floats(B) : work_part_floats(B)) * 4);
     auto cleanup = [&]() {
         for (void* b : bufs) cudaFree(b);
     };
@@ -1036,10 +1052,22 @@ extern "C" cs_status cs_mlp_loss_grad(const float* params, const float* x, const
     cudaMemcpy(p, params, kNParams * 4, cudaMemcpyHostToDevice);
     cudaMemset(g, 0, kNParams * 4);
     cudaMemset(w.loss, 0, 4);
-    round_weights_kernel<<<(kNParams + 255) / 256, 256>>>(p, pr);
-    forward(X, B, pr, w, nullptr);
-    backward(X, T, nullptr, B, pr, g, w, nullptr);
-    cudaError_t e = cudaDeviceSynchronize();
+    cudaError_t e = cudaSuccess;
+    if (fused) {
+        StepArgs sa = {};
+        ReduceArgs ra = {};
+        step_layout(w.part, B, sa, ra);
+        sa.X = X; sa.T = T;
+        sa.p = p;
+        ra.g = g;
+        ra.loss_out = w.loss;
+        if ((e = step_attributes()) == cudaSuccess) step_launch(sa, ra, nullptr);
+    } else {
+        round_weights_kernel<<<(kNParams + 255) / 256, 256>>>(p, pr);
+        forward(X, B, pr, w, nullptr);
+        backward(X, T, nullptr, B, pr, g, w, nullptr);
+    }
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) { set_last_error("mlp gradient", e); cleanup(); return CS_ERR_CUDA; }
     cudaMemcpy(grad, g, kNParams * 4, cudaMemcpyDeviceToHost);
     if (loss) cudaMemcpy(loss, w.loss, 4, cudaMemcpyDeviceToHost);
