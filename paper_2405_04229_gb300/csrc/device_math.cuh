@@ -183,4 +183,22 @@ __device__ __forceinline__ float delta_at(const AtmParams& a, float dz) {
     return a.hom_delta;
 }
 
+// delta_at for heights that only fall from call to call: the layer is kept and
+// left downwards (the same constants and arithmetic).
+struct FallingDelta {
+    float lo, D, c2;   // the layer's bottom and law; above the top: vacuum
+    int i;
+    __device__ __forceinline__ explicit FallingDelta(const AtmParams& a) : lo(a.top_rel), D(0.0f), c2(0.0f), i(a.n_layers) {}
+    __device__ __forceinline__ float at(const AtmParams& a, float dz) {
+        if (a.kind != CS_ATM_LAYERED) return delta_at(a, dz);
+        while (dz < lo) {
+            --i;
+            D = a.lay_D[i];
+            c2 = a.lay_c2[i];
+            lo = i > 0 ? a.lay_lo[i] : -3.0e38f;
+        }
+        return D * ex2_approx(c2 * dz);
+    }
+};
+
 }  // namespace cs
