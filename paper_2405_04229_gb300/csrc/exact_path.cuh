@@ -17,6 +17,8 @@
 // kernel's main path keeps its registers.
 #pragma once
 
+#include <type_traits>
+
 #include "device_math.cuh"
 
 namespace cs {
@@ -49,10 +51,10 @@ __device__ __forceinline__ float next_break(const AtmParams& a, float x) {
     return b;
 }
 
-// End of the sub-interval that starts at x on the way up to dz.
-__device__ __forceinline__ float next_cut(const AtmParams& a, float x, float dz) {
+// End of the sub-interval that starts at x on the way up to dz, `brk` the next breakpoint above x.
+__device__ __forceinline__ float next_cut(float brk, float x, float dz) {
     float c = fminf(x + fmaxf(2000.0f, dz * (1.0f / 128.0f)), dz);
-    c = fminf(c, next_break(a, x));
+    c = fminf(c, brk);
     if (x < 20.0f) c = fminf(c, 20.0f);
     else if (x < 200.0f) c = fminf(c, 200.0f);
     else if (x < 2000.0f) c = fminf(c, 2000.0f);
@@ -65,35 +67,39 @@ __device__ __forceinline__ float next_cut(const AtmParams& a, float x, float dz)
 
 // n - 1 on one piece between breakpoints: d(y) = a 2^(b (y - c)) (layers, table
 // intervals, vacuum with a = 0) or a + b y (linear and homogeneous kinds).  The
-// law is looked up once per sub-interval, at a point inside the piece.
+// law and the next breakpoint are looked up once per piece.
 struct PieceLaw {
     float a, b, c;
-    int linear;
 };
 __device__ __forceinline__ PieceLaw piece_law(const AtmParams& ap, float y) {
     if (ap.kind == CS_ATM_LAYERED) {
-        if (y >= ap.top_rel) return PieceLaw{0.0f, 0.0f, 0.0f, 1};
+        if (y >= ap.top_rel) return PieceLaw{0.0f, 0.0f, 0.0f};
         int i = 0;
         for (int k = 1; k < ap.n_layers; ++k)
             if (y >= ap.lay_lo[k]) i = k;
-        return PieceLaw{ap.lay_D[i], ap.lay_c2[i], 0.0f, 0};
+        return PieceLaw{ap.lay_D[i], ap.lay_c2[i], 0.0f};
     }
     if (ap.kind == CS_ATM_TABLE) {
-        if (y >= ap.top_rel) return PieceLaw{0.0f, 0.0f, 0.0f, 1};
+        if (y >= ap.top_rel) return PieceLaw{0.0f, 0.0f, 0.0f};
         int lo = 0, hi = ap.n_nodes - 1;
         while (hi - lo > 1) {
             const int mid = (lo + hi) >> 1;
             if (__ldg(ap.node_lo + mid) <= y) lo = mid;
             else hi = mid;
         }
-        return PieceLaw{__ldg(ap.node_d + lo), __ldg(ap.node_c2 + lo), __ldg(ap.node_lo + lo), 0};
+        return PieceLaw{__ldg(ap.node_d + lo), __ldg(ap.node_c2 + lo), __ldg(ap.node_lo + lo)};
     }
     if (ap.kind == CS_ATM_LINEAR)
-        return y >= ap.lin_top_rel ? PieceLaw{ap.lin_d1, 0.0f, 0.0f, 1} : PieceLaw{ap.lin_d0, ap.lin_slope, 0.0f, 1};
-    return PieceLaw{ap.hom_delta, 0.0f, 0.0f, 1};
+        return y >= ap.lin_top_rel ? PieceLaw{ap.lin_d1, 0.0f, 0.0f} : PieceLaw{ap.lin_d0, ap.lin_slope, 0.0f};
+    return PieceLaw{ap.hom_delta, 0.0f, 0.0f};
 }
+template <bool LINEAR>
 __device__ __forceinline__ float piece_delta(const PieceLaw& L, float y) {
-    return L.linear ? fmaf(L.b, y, L.a) : L.a * exp2f(L.b * (y - L.c));
+    return LINEAR ? fmaf(L.b, y, L.a) : L.a * ex2_approx(L.b * (y - L.c));
+}
+// Layers and table intervals hold exponential laws (and vacuum) only, the other kinds linear ones only.
+__device__ __forceinline__ bool linear_law(const AtmParams& ap) {
+    return ap.kind != CS_ATM_LAYERED && ap.kind != CS_ATM_TABLE;
 }
 
 // One-sided limit of n - 1 from below at a breakpoint b > 0.
@@ -125,22 +131,27 @@ __device__ __noinline__ float4 exact_fields_planar(const AtmParams* __restrict__
         if (!reaches) return make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
     float aR = 0.0f, aT = 0.0f, aX = 0.0f, aA = 0.0f;
+    auto integrate = [&](auto lin) {
+    float brk = 0.0f;
+    PieceLaw law;
     for (float xa = 0.0f; xa < dz;) {
-        const float xb = next_cut(ap, xa, dz);
+        const bool enter = xa >= brk;   // a new piece
+        if (enter) brk = next_break(ap, xa);
+        const float xb = next_cut(brk, xa, dz);
         const float mid = 0.5f * (xa + xb), half = 0.5f * (xb - xa);
-        const PieceLaw law = piece_law(ap, mid);
+        if (enter) law = piece_law(ap, mid);
         // unrolled: the points' special-function chains overlap (a few photons beyond the
         // tables leave one warp to integrate them, so latency, not issue, sets its time)
 #pragma unroll
         for (int g = 0; g < 16; ++g) {
             const float gx = c_gl16_x[g & 7], y = (g < 8) ? fmaf(-half, gx, mid) : fmaf(half, gx, mid);
             const float wt = half * c_gl16_w[g & 7];
-            const float d = piece_delta(law, y);
+            const float d = piece_delta<decltype(lin)::value>(law, y);
             if (refr) {
                 const float n = 1.0f + d, n2 = n * n;
                 const float D = (d - de) * (2.0f + d + de);
                 const float q2 = fmaxf(fmaf(ne * ne, c2, D), 1e-30f);
-                const float iq = rsqrtf(q2), q = q2 * iq;
+                const float iq = rsqrt_approx(q2), q = q2 * iq;
                 aR = fmaf(wt, -D * iq * rcp_approx(fmaf(ne, c0, q)), aR);
                 aT = fmaf(wt, (c2 * (fmaf(d, d, 2.0f * d) - de) * (n2 + ne) - D) * iq * rcp_approx(fmaf(n2, c0, q)), aT);
                 if (trans) {
@@ -154,6 +165,9 @@ __device__ __noinline__ float4 exact_fields_planar(const AtmParams* __restrict__
         }
         xa = xb;
     }
+    };
+    if (linear_law(ap)) integrate(std::true_type{});
+    else integrate(std::false_type{});
     if (!refr) return make_float4(0.0f, 0.0f, aX, aA);
     return make_float4(c2 * aR, aT, c0 * aX, c0 * aA);
 }
@@ -196,20 +210,25 @@ __device__ __noinline__ float4 exact_fields_sph(const AtmParams* __restrict__ g,
     const float de = refr ? delta_at(ap, dz) : 0.0f;
     const float re = ap.rg + dz, K = (1.0f + de) * re * s0;
     float aP = 0.0f, aT = 0.0f, aX = 0.0f, aA = 0.0f;
+    auto integrate = [&](auto lin) {
+    float brk = 0.0f;
+    PieceLaw law;
     for (float xa = 0.0f; xa < dz;) {
-        const float xb = next_cut(ap, xa, dz);
+        const bool enter = xa >= brk;   // a new piece
+        if (enter) brk = next_break(ap, xa);
+        const float xb = next_cut(brk, xa, dz);
         const float mid = 0.5f * (xa + xb), half = 0.5f * (xb - xa);
-        const PieceLaw law = piece_law(ap, mid);
+        if (enter) law = piece_law(ap, mid);
         // unrolled: the points' special-function chains overlap (a few photons beyond the
         // tables leave one warp to integrate them, so latency, not issue, sets its time)
 #pragma unroll
         for (int g = 0; g < 16; ++g) {
             const float gx = c_gl16_x[g & 7], y = (g < 8) ? fmaf(-half, gx, mid) : fmaf(half, gx, mid);
             const float wt = half * c_gl16_w[g & 7];
-            const float d = (refr || trans) ? piece_delta(law, y) : 0.0f;
+            const float d = (refr || trans) ? piece_delta<decltype(lin)::value>(law, y) : 0.0f;
             const float dg = refr ? d : 0.0f;   // n - 1 in the geometry
             const float r = ap.rg + y, nr = (1.0f + dg) * r;
-            const float iq = rsqrtf(fmaxf(sph_nrK(ap, y, dg, de, dz, om, s0) * (nr + K), 1e-30f));
+            const float iq = rsqrt_approx(fmaxf(sph_nrK(ap, y, dg, de, dz, om, s0) * (nr + K), 1e-30f));
             aP = fmaf(wt, K * iq * rcp_approx(r), aP);
             aT = fmaf(wt, (1.0f + dg) * nr * iq, aT);
             if (trans) {
@@ -219,6 +238,9 @@ __device__ __noinline__ float4 exact_fields_sph(const AtmParams* __restrict__ g,
         }
         xa = xb;
     }
+    };
+    if (linear_law(ap)) integrate(std::true_type{});
+    else integrate(std::false_type{});
     return make_float4(aP, aT, c0 * aX, c0 * aA);
 }
 

@@ -333,6 +333,10 @@ __device__ __forceinline__ int substep(const SM& S, float4& rec, int sg, int k, 
     const float uk = uniform24(rc.x);
     const float fl = floorf(nbar);
     const int N = (int)fl + (uk < nbar - fl ? 1 : 0);
+    if (FL) {   // isotropic: no cone
+        rec = make_float4(0.0f, 0.0f, d, __int_as_float(sg | (k << kKShift)));
+        return N;
+    }
     const float c2 = fmaxf(1.0f - sin2, 1e-30f), s2 = fmaxf(sin2, 1e-30f);
     rec = make_float4(c2 * rsqrt_approx(c2), sin2 > 0.0f ? s2 * rsqrt_approx(s2) : 0.0f, d, __int_as_float(sg | (k << kKShift)));
     return N;
@@ -1308,6 +1312,7 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
         const int lane = t & 31;
         const unsigned int upto = 0xffffffffu >> (31 - lane), below = upto >> 1;   // lanes 0 .. lane, 0 .. lane - 1
         const long long n_wtiles = (pp.n + kWTile - 1) / kWTile;
+        bool q_full = pp.q_cap == 0;   // the queue of bunches beyond the tables takes no more
         // `count` (at most 32) segments from `base` on; of their rounds of 32 bunches, those with
         // index part mod `parts` (a power of two); part 0 counts the segments and what they emit
         auto process_tile = [&](const long long base, const int count, const int part, const int parts) {
@@ -1436,13 +1441,14 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                                 const unsigned int m = __activemask();
                                 const int leader = __ffs(m) - 1;
                                 unsigned int slot0 = 0;
-                                // (a full queue takes no more reservations, so the 32-bit count cannot wrap)
-                                if (lane == leader)
-                                    slot0 = pp.q_cap && __ldcg(scratch + 3) < pp.q_cap ? atomicAdd(scratch + 3, (unsigned int)__popc(m))
-                                                                                       : 0xFFFFFFFFu;
+                                // (a lane that has found the queue full reserves no more: at most 32 entries
+                                // a thread beyond its end, so the 32-bit count cannot wrap.  Reading the count
+                                // first instead costs a second round trip to L2.)
+                                if (lane == leader) slot0 = q_full ? 0xFFFFFFFFu : atomicAdd(scratch + 3, (unsigned int)__popc(m));
+                                q_full = q_full || (lane == leader && slot0 >= pp.q_cap);
                                 slot0 = __shfl_sync(m, slot0, leader);
                                 const unsigned int qslot = slot0 + (unsigned int)__popc(m & below);
-                                if (slot0 != 0xFFFFFFFFu && qslot >= slot0 && qslot < pp.q_cap) {
+                                if (slot0 < pp.q_cap && qslot < pp.q_cap) {
                                     const int segk = __float_as_int(W.sub[j].w);
                                     const unsigned long long li = (unsigned long long)(base + (segk & ((1 << kKShift) - 1)));
                                     reinterpret_cast<uint4*>(scratch + pp.q_off)[qslot] =
@@ -1485,13 +1491,22 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
             }
         };
         if constexpr (!EX) {
-            for (;;) {   // dynamic scheduling: warp tiles (or their parts) from the work counter
+            // dynamic scheduling: warp tiles (or their parts) from the work counter.  (A first tile by the
+            // warp's place in the grid, without the counter, cost two registers and 1-2 % of C2.)
+            for (;;) {
                 unsigned int wt = 0;
                 if (lane == 0) wt = atomicAdd(tile_ctr, 1u);
                 wt = __shfl_sync(0xffffffffu, wt, 0);
                 const long long base = (long long)(TR ? wt >> pp.parts_log2 : wt) * pp.tile_segs;
                 if (base >= pp.n) break;
                 const int part = TR ? (int)(wt & ((1u << pp.parts_log2) - 1u)) : 0;
+                // some warp takes the tile one round of the grid ahead about a tile's time from now:
+                // its segments into L2 (the counter is not advanced: a reserved tile would wait for
+                // a slow warp at the end of the launch)
+                if (!TR) {
+                    const long long ahead = base + (long long)(gridDim.x * (kThreads / 32)) * pp.tile_segs + lane;
+                    if (ahead < pp.n) asm volatile("prefetch.global.L2 [%0];" ::"l"(pp.segs + ahead));
+                }
                 process_tile(base, (int)std::min<long long>(pp.tile_segs, pp.n - base), part, 1 << pp.parts_log2);
             }
         } else {
