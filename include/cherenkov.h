@@ -332,7 +332,7 @@ typedef struct cs_opts {
      * streamed calls through cs_check_timeout). */
     int tc_poll_limit;
     /* Bunches beyond the correction tables are queued by the photon kernel for the exact pass:
-     * entries per warp tile of 32 segments (0 = default 8; at least 4096 and at most 2^22
+     * entries per warp tile of 32 segments (0 = default, 8, of fluorescence 32; at least 4096 and at most 2^22
      * entries in all, and at most the default in the batched and streamed calls; < 0 = no
      * queue).  When the queue is full the remaining such bunches mark their warp tile, which
      * the exact pass then regenerates whole; the results are the same either way. */

@@ -72,6 +72,12 @@ struct AtmParams {
     float lamA_nm;       // aerosol reference wavelength [nm]
     float aer_alpha;
     TableView tv;
+    // the exact path's sub-intervals that do not depend on the photon (see exact_path.cuh): n_gl of
+    // them from the observation level up, gl_end[k] the end of the k-th, 16 points {weight, n - 1,
+    // density x n, aerosol x n} each (layered and tabulated kinds with refraction and transmission)
+    int n_gl;
+    const float* gl_end;
+    const float4* gl_nodes;
     const AtmParams* self;   // device copy of these parameters (for out-of-line routines)
 };
 
@@ -206,6 +212,7 @@ struct cs_atmosphere {
     cs::AtmParams* d_params;   // device copy of p (owned)
     float4* d_tab;         // device table (owned)
     float* d_nodes;        // tabulated kind: interval laws (owned)
+    float4* d_gl;          // the exact path's photon-independent points, then their intervals' ends (owned)
     double h0, dh, dw;
     int device;
     cs::AtmF64 f64;        // the FP64 description the tables were built from

@@ -107,6 +107,30 @@ __device__ __forceinline__ float delta_below(const AtmParams& a, float b) {
     return delta_at(a, __int_as_float(__float_as_int(b) - 1));
 }
 
+// The sub-intervals from the observation level up that next_cut gives whatever
+// the photon, as long as they end at least 2 km below its emission: their ends
+// and points, by the arithmetic of the integration loop below, which reads them
+// instead of forming them anew for every photon (two of a point's five special
+// functions, a third of its instructions).
+constexpr int kGlMax = 256;
+static __global__ void gl_points_kernel(const AtmParams ap, float4* nodes, float* ends, int* count) {
+    const int g = threadIdx.x;   // 16 threads
+    const float gx = c_gl16_x[g & 7];
+    int k = 0;
+    for (float xa = 0.0f; xa < ap.top_rel && k < kGlMax; ++k) {
+        const float xb = next_cut(next_break(ap, xa), xa, 250000.0f);
+        const float mid = 0.5f * (xa + xb), half = 0.5f * (xb - xa);
+        const PieceLaw law = piece_law(ap, mid);
+        const float y = (g < 8) ? fmaf(-half, gx, mid) : fmaf(half, gx, mid);
+        const float d = piece_delta<false>(law, y), n = 1.0f + d;
+        nodes[k * 16 + g] = make_float4(half * c_gl16_w[g & 7], d, ap.rho_per_delta * d * n,
+                                        ap.aer_hobs * ex2_approx(ap.aer_c2 * y) * n);
+        if (g == 0) ends[k] = xb;
+        xa = xb;
+    }
+    if (g == 0) *count = k;
+}
+
 // Planar exact path from dz above the observation level at zenith theta0
 // (c0 = cos theta0 > 0) down to the observation level.  Returns the table
 // fields {G_R, G_t, G_X, G_A} (normalised as the tables store them) and in
@@ -117,7 +141,7 @@ __device__ __forceinline__ float delta_below(const AtmParams& a, float b) {
 //   dR / sin(theta0) * cos(theta0) = -D / (q (n_e c0 + q))
 //   c dt cos(theta0) = (n^2 c0 - q) / q = [c0^2 (2d + d^2 - d_e)(n^2 + n_e) - D] / (q (n^2 c0 + q))
 //   X = 100 rho n / q,  A = exp(-h / H_A) n / q   (n = 1, q = c0 for the straight line)
-__device__ __noinline__ float4 exact_fields_planar(const AtmParams* __restrict__ g, float dz, float c0, bool& reaches) {
+static __device__ __noinline__ float4 exact_fields_planar(const AtmParams* __restrict__ g, float dz, float c0, bool& reaches) {
     const AtmParams& ap = *g;
     const bool refr = ap.refraction != 0, trans = ap.transmission != 0;
     const float c2 = c0 * c0;
@@ -131,10 +155,32 @@ __device__ __noinline__ float4 exact_fields_planar(const AtmParams* __restrict__
         if (!reaches) return make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
     float aR = 0.0f, aT = 0.0f, aX = 0.0f, aA = 0.0f;
+    float x0 = 0.0f;
+    // (2 km sub-intervals: the photon is not emitted above 256 km)
+    const int n_gl = dz <= 256000.0f ? ap.n_gl : 0;
+    for (int k = 0; k < n_gl; ++k) {
+        const float xb = __ldg(ap.gl_end + k);
+        if (!(xb <= dz - 2000.0f)) break;
+        const float4* p = ap.gl_nodes + k * 16;
+#pragma unroll
+        for (int g = 0; g < 16; ++g) {
+            const float4 v = __ldg(p + g);
+            const float wt = v.x, d = v.y;
+            const float n = 1.0f + d, n2 = n * n;
+            const float D = (d - de) * (2.0f + d + de);
+            const float q2 = fmaxf(fmaf(ne * ne, c2, D), 1e-30f);
+            const float iq = rsqrt_approx(q2), q = q2 * iq;
+            aR = fmaf(wt, -D * iq * rcp_approx(fmaf(ne, c0, q)), aR);
+            aT = fmaf(wt, (c2 * (fmaf(d, d, 2.0f * d) - de) * (n2 + ne) - D) * iq * rcp_approx(fmaf(n2, c0, q)), aT);
+            aX = fmaf(wt, v.z * iq, aX);
+            aA = fmaf(wt, v.w * iq, aA);
+        }
+        x0 = xb;
+    }
     auto integrate = [&](auto lin) {
     float brk = 0.0f;
     PieceLaw law;
-    for (float xa = 0.0f; xa < dz;) {
+    for (float xa = x0; xa < dz;) {
         const bool enter = xa >= brk;   // a new piece
         if (enter) brk = next_break(ap, xa);
         const float xb = next_cut(brk, xa, dz);
@@ -189,7 +235,7 @@ __device__ __forceinline__ float sph_nrK(const AtmParams& ap, float y, float d, 
     return fmaf(rg * om, 1.0f + de, dz * om) + fmaf(rg, d - de, y - dz) + fmaf(d, y, -de * dz * s0);
 }
 
-__device__ __noinline__ bool sph_reaches(const AtmParams* __restrict__ g, float dz, float c0, float s0) {
+static __device__ __noinline__ bool sph_reaches(const AtmParams* __restrict__ g, float dz, float c0, float s0) {
     const AtmParams& ap = *g;
     const float om = c0 * c0 / (1.0f + s0);
     if (!ap.refraction) return sph_nrK(ap, 0.0f, 0.0f, 0.0f, dz, om, s0) > 0.0f;
@@ -203,7 +249,7 @@ __device__ __noinline__ bool sph_reaches(const AtmParams* __restrict__ g, float 
 
 // Returns {Phi [rad], c t_path [m], G_X = X c0, G_A = A c0}; call only for
 // paths that reach the ground (sph_reaches).
-__device__ __noinline__ float4 exact_fields_sph(const AtmParams* __restrict__ g, float dz, float c0, float s0) {
+static __device__ __noinline__ float4 exact_fields_sph(const AtmParams* __restrict__ g, float dz, float c0, float s0) {
     const AtmParams& ap = *g;
     const bool refr = ap.refraction != 0, trans = ap.transmission != 0;
     const float om = c0 * c0 / (1.0f + s0);

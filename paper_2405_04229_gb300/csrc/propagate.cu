@@ -2075,7 +2075,10 @@ cs_status launch(const cs_segment* d_segs, size_t n, const cs_atmosphere* atm, c
     const unsigned int grid = plan_launch(pp, n, o);
     pp.tiles_per_bit = 1;
     const long long n_wtiles = (pp.n + kWTile - 1) / kWTile;
-    pp.q_cap = queue_cap(n_wtiles, o.exact_queue);
+    // fluorescence leaves a quarter of its bunches to the exact pass, 19 a tile at bunch 1: a queue of
+    // eight a tile overflows there, and the pass then regenerates nearly every tile (2e6 segments of
+    // bunch 1: 1533 us, with 32 a tile 966 us)
+    pp.q_cap = queue_cap(n_wtiles, o.exact_queue == 0 && o.emission ? 32 : o.exact_queue);
     pp.q_off = (unsigned int)scratch_queue_off(n_wtiles, 1);
     const size_t bytes = scratch_words(n_wtiles, 1, pp.q_cap) * sizeof(unsigned int);
     unsigned int* scratch = nullptr;

@@ -10,7 +10,7 @@
 
 #include <vector>
 
-#include "common.cuh"
+#include "exact_path.cuh"
 
 namespace cs {
 namespace {
@@ -493,7 +493,7 @@ extern "C" cs_status cs_atmosphere_create(const cs_atmosphere_desc* d, cs_atmosp
     auto fail = [&](const char* where) {
         set_last_error(where, e);
         cudaFree(dF); cudaFree(dFb); cudaFree(dslot); cudaFree(drows); cudaFree(h->d_tab); cudaFree(h->d_nodes);
-        cudaFree(h->d_params);
+        cudaFree(h->d_params); cudaFree(h->d_gl);
         delete h;
         return CS_ERR_CUDA;
     };
@@ -519,6 +519,17 @@ extern "C" cs_status cs_atmosphere_create(const cs_atmosphere_desc* d, cs_atmosp
     p.tv.tab = h->d_tab;
     if ((e = cudaMalloc(&h->d_params, sizeof(AtmParams))) != cudaSuccess) return fail("parameters");
     p.self = h->d_params;
+    // the exact path's photon-independent points
+    if ((a.kind == CS_ATM_LAYERED || a.kind == CS_ATM_TABLE) && p.refraction && p.transmission && !p.spherical) {
+        if ((e = cudaMalloc(&h->d_gl, kGlMax * (16 * sizeof(float4) + sizeof(float)) + sizeof(int))) != cudaSuccess) return fail("exact path");
+        float* ends = (float*)(h->d_gl + kGlMax * 16);
+        int* count = (int*)(ends + kGlMax);
+        gl_points_kernel<<<1, 16>>>(p, h->d_gl, ends, count);
+        if ((e = cudaGetLastError()) != cudaSuccess) return fail("exact path");
+        if ((e = cudaMemcpy(&p.n_gl, count, sizeof(int), cudaMemcpyDeviceToHost)) != cudaSuccess) return fail("exact path");
+        p.gl_end = ends;
+        p.gl_nodes = h->d_gl;
+    }
     if ((e = cudaMemcpy(h->d_params, &p, sizeof(AtmParams), cudaMemcpyHostToDevice)) != cudaSuccess) return fail("parameters");
     *out = h;
     return CS_OK;
@@ -545,6 +556,7 @@ extern "C" void cs_atmosphere_destroy(cs_atmosphere* atm) {
     cudaFree(atm->d_tab);
     cudaFree(atm->d_nodes);
     cudaFree(atm->d_params);
+    cudaFree(atm->d_gl);
     delete atm;
 }
 
