@@ -212,6 +212,9 @@ struct cs_atmosphere {
     cs::AtmParams* d_params;   // device copy of p (owned)
     float4* d_tab;         // device table (owned)
     float* d_nodes;        // tabulated kind: interval laws (owned)
+    int n_pieces;          // FP64 points of the pieces between breakpoints (owned; see tables.cu)
+    int* d_piece_begin;
+    void* d_pieces;
     float4* d_gl;          // the exact path's photon-independent points, then their intervals' ends (owned)
     double h0, dh, dw;
     int device;
