@@ -542,14 +542,20 @@ cs_status alloc(void** p, size_t bytes) {
 
 // Evaluates the trained network through the photon kernel's warp-level
 // inference path on arbitrary (dz, cos(theta0), 1/lambda_nm) inputs.
+//
+// Bound by latency: a row's three MMA round trips and 192 tanh leave little to
+// overlap within a warp, so what counts is warps per SM.  Two blocks of 512
+// threads (64 registers; one block where the split activations need their lo
+// tiles) instead of one of 256: 1e6 points EVAL_MS.
+constexpr int kEvalThreads = 512;
 template <bool SPLIT>
-__global__ void __launch_bounds__(256, 1)
+__global__ void __launch_bounds__(kEvalThreads, SPLIT ? 1 : 2)
 eval_kernel(SurrogateView sv, const float4* __restrict__ in, size_t n, float4* __restrict__ out, int network_only) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    TcSmem<2>& T = *reinterpret_cast<TcSmem<2>*>(smem_raw);
+    TcSmem<kEvalThreads / 128>& T = *reinterpret_cast<TcSmem<kEvalThreads / 128>*>(smem_raw);
     tc_setup(T, sv);
-    // every thread of the block takes the same number of 256-row rounds
-    for (size_t base = (size_t)blockIdx.x * 256; base < n; base += (size_t)gridDim.x * 256) {
+    // every thread of the block takes the same number of rounds
+    for (size_t base = (size_t)blockIdx.x * kEvalThreads; base < n; base += (size_t)gridDim.x * kEvalThreads) {
         const size_t i = base + threadIdx.x;
         const float4 v = i < n ? in[i] : make_float4(0.f, 1.f, 3.0e-3f, 0.f);   // dz, cos(theta0), 1/lambda_nm
         const float x[3] = {sv.in_scale[0] * height_coordinate(sv, v.x) + sv.in_shift[0],
@@ -575,15 +581,18 @@ eval_kernel(SurrogateView sv, const float4* __restrict__ in, size_t n, float4* _
 cs_status run_eval(const SurrogateView& sv, const float4* d_in, size_t n, float4* d_out, cudaStream_t s,
                    int network_only = 0) {
     if (n == 0) return CS_OK;
-    const int smem = (int)sizeof(TcSmem<2>);
-    CS_CUDA_TRY(cudaFuncSetAttribute(eval_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    CS_CUDA_TRY(cudaFuncSetAttribute(eval_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    const unsigned grid = (unsigned)std::min<size_t>((n + 255) / 256, (size_t)device_sm_count());
-    if (sv.split) eval_kernel<true><<<grid, 256, smem, s>>>(sv, d_in, n, d_out, network_only);
-    else eval_kernel<false><<<grid, 256, smem, s>>>(sv, d_in, n, d_out, network_only);
+    const bool split = sv.split != 0;
+    const int smem = (int)TcSmem<kEvalThreads / 128>::bytes(split);
+    CS_CUDA_TRY(cudaFuncSetAttribute(split ? eval_kernel<true> : eval_kernel<false>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    const unsigned grid = (unsigned)std::min<size_t>((n + kEvalThreads - 1) / kEvalThreads,
+                                                     (size_t)device_sm_count() * (split ? 1 : 2));
+    if (split) eval_kernel<true><<<grid, kEvalThreads, smem, s>>>(sv, d_in, n, d_out, network_only);
+    else eval_kernel<false><<<grid, kEvalThreads, smem, s>>>(sv, d_in, n, d_out, network_only);
     CS_CUDA_TRY(cudaGetLastError());
+    const bool timed_out = tc_take_timeout(s);
     CS_CUDA_TRY(cudaStreamSynchronize(s));
-    return tc_take_timeout() ? CS_ERR_TIMEOUT : CS_OK;
+    return timed_out ? CS_ERR_TIMEOUT : CS_OK;
 }
 
 }  // namespace

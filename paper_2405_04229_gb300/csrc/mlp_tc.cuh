@@ -21,11 +21,13 @@ constexpr int kTcSpin = 1 << 20;                     // polls of an MMA completi
 
 // Shared memory of the tensor-core network, per CTA of NWG warpgroups; the
 // CTA holds NWG x 64 tensor-memory columns (64 FP32 accumulators per row).
+// The tiles of the activations' lo parts follow it where the network splits
+// them (bytes()); without them two evaluation blocks fit an SM.
 template <int NWG>
 struct TcSmem {
     static_assert(NWG == 2 || NWG == 4, "tensor-memory allocations are powers of two >= 32 columns");
     static constexpr unsigned int kCols = 64 * NWG;
-    __align__(128) unsigned char a[NWG][2][kTcATile];  // [warpgroup][hi, lo] activations
+    __align__(128) unsigned char a[NWG][kTcATile];     // activations (hi parts)
     __align__(128) unsigned char w[kTcWBytes];         // BF16 weights, core-matrix layout
     float4 w1p[kHid / 2][2];                           // layer 1, units 2i and 2i + 1 side by side:
                                                        // {W1[.][0], W1[.][1]}, {W1[.][2], b1[.]}
@@ -35,15 +37,19 @@ struct TcSmem {
     unsigned int tmem_base;
     int abort[NWG];                                    // a wait ran out (per warpgroup)
     unsigned int phase[NWG];                           // parity of the next completion
+    __device__ __forceinline__ unsigned char* a_lo(int wg) { return reinterpret_cast<unsigned char*>(this + 1) + wg * kTcATile; }
+    __host__ __device__ static constexpr size_t bytes(bool split) { return sizeof(TcSmem) + (split ? (size_t)NWG * kTcATile : 0); }
 };
 
 // Set when a tensor-core wait ran out (one flag per translation unit); read
 // and cleared by that unit's host calls through tc_take_timeout().
 static __device__ unsigned int g_tc_timeout = 0;
 
-static inline bool tc_take_timeout() {
+static inline bool tc_take_timeout(cudaStream_t s = nullptr) {   // (waits for the stream's work)
     unsigned int v = 0;
-    if (cudaMemcpyFromSymbol(&v, g_tc_timeout, sizeof v) != cudaSuccess) return false;
+    if (cudaMemcpyFromSymbolAsync(&v, g_tc_timeout, sizeof v, 0, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaStreamSynchronize(s) != cudaSuccess)
+        return false;
     if (v) {
         const unsigned int z = 0;
         cudaMemcpyToSymbol(g_tc_timeout, &z, sizeof z);
@@ -248,8 +254,8 @@ __device__ __forceinline__ bool net128_tc(const SurrogateView& sv, TcSmem<NWG>& 
     const int wg = threadIdx.x >> 7, row = threadIdx.x & 127;
     y[0] = y[1] = y[2] = 0.0f;
     if (T.abort[wg]) return false;   // uniform: set before one of this warpgroup's barriers
-    unsigned char* a_hi = T.a[wg][0];
-    unsigned char* a_lo = T.a[wg][1];
+    unsigned char* a_hi = T.a[wg];
+    unsigned char* a_lo = SPLIT ? T.a_lo(wg) : nullptr;
     // layer 1 (3 inputs): FP32 on the CUDA cores
 #pragma unroll 1
     for (int g = 0; g < 8; ++g) {

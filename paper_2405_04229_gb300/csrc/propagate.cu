@@ -81,7 +81,7 @@ static_assert(4 * (kSmemPass + 1024) <= 228 * 1024, "four exact-tracer blocks pe
 
 // The surrogate instances keep the tensor-core network's buffers after the tile.
 constexpr size_t kTcSmemOffset = (sizeof(TileSmem) + 127) & ~(size_t)127;
-constexpr size_t kSmemSurrogate = kTcSmemOffset + sizeof(TcSmem<kThreadsSur / 128>);
+constexpr size_t smem_surrogate(bool split) { return kTcSmemOffset + TcSmem<kThreadsSur / 128>::bytes(split); }
 
 // Exclusive block scan with one barrier; `buf` alternates between calls so a
 // scan never overwrites warp sums another warp may still be reading.
@@ -1718,11 +1718,12 @@ bool compatible(const cs_atmosphere* atm, const cs_detector* det) {
 cs_status launch_kernel(unsigned grid, cudaStream_t stream, const PropParams& pp, const AtmParams& ap,
                         const DetParams& dp, const OutParams& op, unsigned int* ctr, const cs_surrogate* sur,
                         int tc_poll_limit) {
-    const size_t smem = sur ? kSmemSurrogate : kSmemExact;
+    size_t smem = kSmemExact;
     SurrogateView sv;
     memset(&sv, 0, sizeof sv);
     if (sur) {
         sv = *surrogate_view(sur);
+        smem = smem_surrogate(sv.split != 0);
         sv.polls = tc_poll_limit == 0 ? kTcSpin : std::max(tc_poll_limit, 0);
     }
     // outside a stream capture, as programmatic dependent launches: the photon kernel's launch
@@ -1825,7 +1826,7 @@ cs_status set_smem_attributes() {
     if (dev < 0 || dev >= kMaxDevices) return CS_ERR_INVALID_ARG;
     std::lock_guard<std::mutex> lock(g_attr_mu);
     if (g_attr_done[dev]) return CS_OK;
-    const int smem = (int)kSmemExact, smem_sur = (int)kSmemSurrogate;
+    const int smem = (int)kSmemExact, smem_sur = (int)smem_surrogate(true);
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
     CS_CUDA_TRY((set_exact_smem<false, false, false>(smem)));
     CS_CUDA_TRY((set_exact_smem<false, false, true>(smem)));
