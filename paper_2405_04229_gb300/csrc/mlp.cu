@@ -22,7 +22,7 @@ struct cs_surrogate {
     float* d_p = nullptr;             // FP32 master parameters
     __nv_bfloat16* d_wb = nullptr;    // BF16 tensor-core weights
     float4* d_base = nullptr;         // first-order baseline table (see surrogate_baseline)
-    cs::SurrogateView view{};
+    cs::SurrogateNet view{};
     cs_surrogate_stats stats{};
     double h_min = 0, h_max = 0, theta_max = 0, lambda_min = 0, lambda_max = 0;
 };
@@ -550,7 +550,7 @@ cs_status alloc(void** p, size_t bytes) {
 constexpr int kEvalThreads = 512;
 template <bool SPLIT>
 __global__ void __launch_bounds__(kEvalThreads, SPLIT ? 1 : 2)
-eval_kernel(SurrogateView sv, const float4* __restrict__ in, size_t n, float4* __restrict__ out, int network_only) {
+eval_kernel(const __grid_constant__ SurrogateNet sv, const float4* __restrict__ in, size_t n, float4* __restrict__ out, int network_only) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     TcSmem<kEvalThreads / 128>& T = *reinterpret_cast<TcSmem<kEvalThreads / 128>*>(smem_raw);
     tc_setup(T, sv);
@@ -578,7 +578,7 @@ eval_kernel(SurrogateView sv, const float4* __restrict__ in, size_t n, float4* _
 
 // The network on n inputs through the tensor-core path, synchronously;
 // CS_ERR_TIMEOUT if a wait on the tensor cores ran out.
-cs_status run_eval(const SurrogateView& sv, const float4* d_in, size_t n, float4* d_out, cudaStream_t s,
+cs_status run_eval(const SurrogateNet& sv, const float4* d_in, size_t n, float4* d_out, cudaStream_t s,
                    int network_only = 0) {
     if (n == 0) return CS_OK;
     const bool split = sv.split != 0;
@@ -599,7 +599,7 @@ cs_status run_eval(const SurrogateView& sv, const float4* d_in, size_t n, float4
 }  // namespace cs
 
 namespace cs {
-const SurrogateView* surrogate_view(const cs_surrogate* s) { return &s->view; }
+const SurrogateNet* surrogate_view(const cs_surrogate* s) { return &s->view; }
 }  // namespace cs
 
 using namespace cs;
@@ -906,8 +906,17 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
     }
     round_weights_kernel<<<(kNParams + 255) / 256, 256, 0, s>>>(p, sg->d_p);
     to_bf16_kernel<<<(kNBf16 + 255) / 256, 256, 0, s>>>(p, sg->d_wb);
-    SurrogateView& sv = sg->view;
-    sv = bv;   // the baseline table and constants
+    SurrogateNet& sv = sg->view;
+    static_cast<SurrogateView&>(sv) = bv;   // the baseline table and constants
+    e = cudaMemcpy(hp.data(), p, kNParams * 4, cudaMemcpyDeviceToHost);
+    for (int i = 0; i < kHid / 2; ++i) {
+        const float *w = hp.data() + kOffW1 + 6 * i, *b = hp.data() + kOffB1 + 2 * i;
+        sv.w1p[i][0] = make_float4(w[0], w[3], w[1], w[4]);
+        sv.w1p[i][1] = make_float4(w[2], w[5], b[0], b[1]);
+    }
+    memcpy(sv.b23[0], hp.data() + kOffB2, sizeof sv.b23[0]);
+    memcpy(sv.b23[1], hp.data() + kOffB3, sizeof sv.b23[1]);
+    for (int k = 0; k < 4; ++k) sv.b4[k] = k < kNOut ? hp[kOffB4 + k] : 0.0f;
     sv.p = sg->d_p;
     sv.wb = sg->d_wb;
     sv.split = cfg.split_activations ? 1 : 0;

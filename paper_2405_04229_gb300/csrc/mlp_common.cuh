@@ -61,6 +61,16 @@ struct SurrogateView {
     int polls;   // polls of each tensor-core completion before giving up (>= 0)
 };
 
+// The view with the parameters that every thread reads at the same time, as kernel parameters: read
+// through the constant cache as operands.  (From shared memory their 96 16-byte loads a row took
+// about half of the SM's shared-memory cycles.)
+struct SurrogateNet : SurrogateView {
+    float4 w1p[kHid / 2][2];   // layer 1, units 2i and 2i + 1 side by side:
+                               // {W1[.][0], W1[.][1]}, {W1[.][2], b1[.]}
+    float4 b23[2][kHid / 4];   // biases of layers 2 and 3
+    float b4[4];
+};
+
 __device__ __forceinline__ float height_coordinate(const SurrogateView& sv, float dz) {
     return sv.inv_height_scale > 0.0f ? ex2_approx(-dz * sv.inv_height_scale * 1.4426950408889634f) : dz;
 }
@@ -98,7 +108,7 @@ __device__ __forceinline__ float3 surrogate_baseline(const SurrogateView& sv, fl
 }
 
 // The trained network's view (defined with the training code).
-const SurrogateView* surrogate_view(const cs_surrogate* s);
+const SurrogateNet* surrogate_view(const cs_surrogate* s);
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);

@@ -29,10 +29,6 @@ struct TcSmem {
     static constexpr unsigned int kCols = 64 * NWG;
     __align__(128) unsigned char a[NWG][kTcATile];     // activations (hi parts)
     __align__(128) unsigned char w[kTcWBytes];         // BF16 weights, core-matrix layout
-    float4 w1p[kHid / 2][2];                           // layer 1, units 2i and 2i + 1 side by side:
-                                                       // {W1[.][0], W1[.][1]}, {W1[.][2], b1[.]}
-    float4 b23[2][kHid / 4];                           // biases of layers 2 and 3
-    float b4[4];
     unsigned long long mbar[NWG];                      // MMA completion, per warpgroup
     unsigned int tmem_base;
     int abort[NWG];                                    // a wait ran out (per warpgroup)
@@ -208,15 +204,6 @@ __device__ __forceinline__ void tc_setup(TcSmem<NWG>& T, const SurrogateView& sv
         }
         *reinterpret_cast<uint4*>(T.w + dst) = v;
     }
-    const float* p = sv.p;
-    for (int i = t; i < kHid / 2; i += blockDim.x) {
-        const int u = 2 * i, v = u + 1;
-        T.w1p[i][0] = make_float4(p[kOffW1 + 3 * u], p[kOffW1 + 3 * v], p[kOffW1 + 3 * u + 1], p[kOffW1 + 3 * v + 1]);
-        T.w1p[i][1] = make_float4(p[kOffW1 + 3 * u + 2], p[kOffW1 + 3 * v + 2], p[kOffB1 + u], p[kOffB1 + v]);
-    }
-    for (int i = t; i < 2 * kHid; i += blockDim.x)
-        reinterpret_cast<float*>(T.b23)[i] = p[(i < kHid ? kOffB2 : kOffB3 - kHid) + i];
-    if (t < 4) T.b4[t] = t < kNOut ? p[kOffB4 + t] : 0.0f;
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
@@ -250,21 +237,21 @@ __device__ __forceinline__ void tc_teardown(TcSmem<NWG>& T) {
 // threads of the warpgroup call it together.  Returns false (outputs zero)
 // once a wait of this warpgroup has run out.
 template <bool SPLIT, int NWG>
-__device__ __forceinline__ bool net128_tc(const SurrogateView& sv, TcSmem<NWG>& T, const float (&x)[3], float (&y)[3]) {
+__device__ __forceinline__ bool net128_tc(const SurrogateNet& sv, TcSmem<NWG>& T, const float (&x)[3], float (&y)[3]) {
     const int wg = threadIdx.x >> 7, row = threadIdx.x & 127;
     y[0] = y[1] = y[2] = 0.0f;
     if (T.abort[wg]) return false;   // uniform: set before one of this warpgroup's barriers
     unsigned char* a_hi = T.a[wg];
     unsigned char* a_lo = SPLIT ? T.a_lo(wg) : nullptr;
     // layer 1 (3 inputs): FP32 on the CUDA cores
-#pragma unroll 1
+#pragma unroll
     for (int g = 0; g < 8; ++g) {
         float h[8];
         // two units per packed FP32 instruction (the same fused operations in the same order)
         const float2 x0 = make_float2(x[0], x[0]), x1 = make_float2(x[1], x[1]), x2 = make_float2(x[2], x[2]);
 #pragma unroll
         for (int j = 0; j < 8; j += 2) {
-            const float4 wa = T.w1p[(8 * g + j) >> 1][0], wb = T.w1p[(8 * g + j) >> 1][1];
+            const float4 wa = sv.w1p[(8 * g + j) >> 1][0], wb = sv.w1p[(8 * g + j) >> 1][1];
             float2 z = __ffma2_rn(make_float2(wa.x, wa.y), x0, make_float2(wb.z, wb.w));
             z = __ffma2_rn(make_float2(wa.z, wa.w), x1, z);
             z = __ffma2_rn(make_float2(wb.x, wb.y), x2, z);
@@ -281,7 +268,7 @@ __device__ __forceinline__ bool net128_tc(const SurrogateView& sv, TcSmem<NWG>& 
     const uint32_t d_tmem = T.tmem_base + (uint32_t)(wg * kHid);
     const uint32_t t_lane = d_tmem + ((uint32_t)(((threadIdx.x >> 5) & 3) * 32) << 16);
     const uint32_t mbar = smem_u32(&T.mbar[wg]);
-#pragma unroll 1
+#pragma unroll
     for (int L = 0; L < 3; ++L) {
         // the operand tile is complete and earlier reads of the accumulators are done
         fence_async_smem();
@@ -308,8 +295,8 @@ __device__ __forceinline__ bool net128_tc(const SurrogateView& sv, TcSmem<NWG>& 
         if (T.abort[wg]) return false;
         tc_fence_after();
         if (L < 2) {
-            const float4* bias = T.b23[L];
-#pragma unroll 1
+            const float4* bias = sv.b23[L];
+#pragma unroll
             for (int c = 0; c < kHid / 16; ++c) {
                 float v[16];
                 tc_ld16(t_lane + (uint32_t)(16 * c), v);
@@ -348,7 +335,7 @@ __device__ __forceinline__ bool net128_tc(const SurrogateView& sv, TcSmem<NWG>& 
             float v[4];
             tc_ld4(t_lane, v);
 #pragma unroll
-            for (int k = 0; k < 3; ++k) y[k] = v[k] + T.b4[k];
+            for (int k = 0; k < 3; ++k) y[k] = v[k] + sv.b4[k];
         }
     }
     tc_fence_before();   // these accumulator reads precede the next call's MMAs (its barrier)

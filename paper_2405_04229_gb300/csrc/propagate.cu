@@ -700,6 +700,11 @@ __device__ __forceinline__ void correction_fields(const AtmParams& ap, bool use_
     if (!(FIX || ap.transmission)) Tr = 1.0f;
 }
 
+// The network as a kernel parameter, nothing in the other instances.
+struct NoNet {};
+template <bool SURR>
+using NetParam = std::conditional_t<SURR, SurrogateNet, NoNet>;
+
 // Stages 3-5 for one bunch: generation on the cone (Sec. 4.2), the upward
 // filter (Sec. 5.3.4), straight line (Eq. 3.3; on the sphere, the vacuum
 // line to the ground sphere) plus the interpolation-tracing correction
@@ -717,7 +722,7 @@ enum { kModeMain = 0, kModeCheck = 1, kModeExact = 2 };
 template <bool SURR, bool SPH, bool REC, bool FL, bool TR, int MODE = kModeMain, bool FIX = false, typename SM>
 __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, long long base,
                                       const PropParams& pp, const AtmParams& ap, const DetParams& dp,
-                                      const OutParams& op, const SurrogateView& sv, TcSmem<kThreadsSur / 128>* tcs,
+                                      const OutParams& op, const NetParam<SURR>& sv, TcSmem<kThreadsSur / 128>* tcs,
                                       Tally& T) {
     // The launch configuration; FIX instances are launched only for the standard one (refraction,
     // transmission and tables on; histogram, telescopes and time sums on; no camera optics), where
@@ -802,7 +807,7 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
     // ---- the surrogate network, warp-collective --------------------------------
     float net[3] = {0.0f, 0.0f, 1.0f};
     bool use_net = false;
-    if (SURR) {
+    if constexpr (SURR) {
         use_net = active && status == CS_ST_LANDED && in_surrogate_domain(sv, dz, cos_z);
         const float x[3] = {use_net ? fmaf(sv.in_scale[0], height_coordinate(sv, dz), sv.in_shift[0]) : 0.0f,
                             use_net ? fmaf(sv.in_scale[1], cos_z, sv.in_shift[1]) : 0.0f,
@@ -1284,7 +1289,7 @@ template <bool SURR, bool SPH, int MINB, bool REC, bool FL = false, bool TR = fa
           bool FIX = false, int NT = SURR ? kThreadsSur : kThreads>
 __global__ void __launch_bounds__(NT, MINB)
 propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, const OutParams op,
-                 unsigned int* scratch, const SurrogateView sv) {
+                 unsigned int* scratch, const NetParam<SURR> sv) {
     static_assert(!(EX && SURR), "the exact pass runs the exact-tracer form");
     // The photon kernel is launched as a programmatic dependent of the kernel that zeroes its outputs
     // and scratch, the exact pass as one of the photon kernel: its blocks become resident as the
@@ -1299,7 +1304,7 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
     TileSmem& S = *reinterpret_cast<TileSmem*>(smem_raw);
     TcSmem<kThreadsSur / 128>* tcs = SURR ? reinterpret_cast<TcSmem<kThreadsSur / 128>*>(smem_raw + kTcSmemOffset) : nullptr;
     const int t = threadIdx.x;
-    if (SURR) tc_setup(*tcs, sv);
+    if constexpr (SURR) tc_setup(*tcs, sv);
     const long long n_tiles = (pp.n + kTile - 1) / kTile;
     unsigned int emitted = 0, invalid = 0, dropped = 0;
     Tally T = {0, 0, 0, 0};
@@ -1719,19 +1724,18 @@ cs_status launch_kernel(unsigned grid, cudaStream_t stream, const PropParams& pp
                         const DetParams& dp, const OutParams& op, unsigned int* ctr, const cs_surrogate* sur,
                         int tc_poll_limit) {
     size_t smem = kSmemExact;
-    SurrogateView sv;
-    memset(&sv, 0, sizeof sv);
+    SurrogateNet net;
     if (sur) {
-        sv = *surrogate_view(sur);
-        smem = smem_surrogate(sv.split != 0);
-        sv.polls = tc_poll_limit == 0 ? kTcSpin : std::max(tc_poll_limit, 0);
+        net = *surrogate_view(sur);
+        smem = smem_surrogate(net.split != 0);
+        net.polls = tc_poll_limit == 0 ? kTcSpin : std::max(tc_poll_limit, 0);
     }
     // outside a stream capture, as programmatic dependent launches: the photon kernel's launch
     // overlaps the zeroing before it, the exact pass's the photon kernel's tail (for most workloads
     // the pass finds nothing to do)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     CS_CUDA_TRY(cudaStreamIsCapturing(stream, &cap));
-    auto dependent = [&](auto kernel, unsigned int blocks, int threads, size_t bytes) {
+    auto dependent = [&](auto kernel, unsigned int blocks, int threads, size_t bytes, const auto& sv) {
         if (cap == cudaStreamCaptureStatusNone) {
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3(blocks);
@@ -1749,7 +1753,8 @@ cs_status launch_kernel(unsigned grid, cudaStream_t stream, const PropParams& pp
         kernel<<<blocks, threads, bytes, stream>>>(pp, ap, dp, op, ctr, sv);
     };
     // instances: (network or tables) x (sphere or plane) x (records or throughput)
-    auto go = [&](auto kernel, int threads) { dependent(kernel, grid, threads, smem); };
+    auto go = [&](auto kernel, int threads) { dependent(kernel, grid, threads, smem, NoNet{}); };
+    auto go_net = [&](auto kernel) { dependent(kernel, grid, kThreadsSur, smem, net); };
     const bool rec = op.records != nullptr;
     // the exact tracer's instances: emission (Cherenkov or fluorescence) x tracer (tables or stepper)
     // the standard configuration (refraction, transmission and tables; histogram, telescopes and
@@ -1771,8 +1776,8 @@ cs_status launch_kernel(unsigned grid, cudaStream_t stream, const PropParams& pp
     using f_ = std::false_type;
     const bool fl = pp.emission != 0, tr = pp.snell != 0;
     if (sur) {
-        if (ap.spherical) rec ? go(propagate_kernel<true, true, 1, true>, kThreadsSur) : go(propagate_kernel<true, true, 1, false>, kThreadsSur);
-        else rec ? go(propagate_kernel<true, false, 1, true>, kThreadsSur) : go(propagate_kernel<true, false, 1, false>, kThreadsSur);
+        if (ap.spherical) rec ? go_net(propagate_kernel<true, true, 1, true>) : go_net(propagate_kernel<true, true, 1, false>);
+        else rec ? go_net(propagate_kernel<true, false, 1, true>) : go_net(propagate_kernel<true, false, 1, false>);
     } else if (ap.spherical) {
         if (fl) tr ? exact(t_{}, t_{}, t_{}) : exact(t_{}, t_{}, f_{});
         else tr ? exact(t_{}, f_{}, t_{}) : exact(t_{}, f_{}, f_{});
@@ -1786,7 +1791,7 @@ cs_status launch_kernel(unsigned grid, cudaStream_t stream, const PropParams& pp
     if (ap.use_tables && !(tr && ap.refraction)) {
         const long long n_wtiles = (pp.n + kWTile - 1) / kWTile;
         const unsigned grid_x = (unsigned)std::max<long long>(1, std::min<long long>(n_wtiles, (long long)device_sm_count() * 4));
-        auto pass = [&](auto kernel) { dependent(kernel, grid_x, kThreads, kSmemPass); };
+        auto pass = [&](auto kernel) { dependent(kernel, grid_x, kThreads, kSmemPass, NoNet{}); };
         if (ap.spherical) {
             if (fl) rec ? pass(propagate_kernel<false, true, 4, true, true, false, true>) : pass(propagate_kernel<false, true, 4, false, true, false, true>);
             else rec ? pass(propagate_kernel<false, true, 4, true, false, false, true>) : pass(propagate_kernel<false, true, 4, false, false, false, true>);
