@@ -288,8 +288,8 @@ __device__ __forceinline__ int import_segment(SM& S, int t, const cs_segment* se
     S.z2[t] = (FL ? pp.fl_yd : ap.ft) * (z * z);
     S.shower[t] = (int)shower;
     const int bsz = pp.shower_bunch ? __ldg(pp.shower_bunch + shower) : pp.bunch;
-        S.bunch[t] = bsz;
-        S.inv_b[t] = rcp_approx((float)bsz);
+    S.bunch[t] = bsz;
+    S.inv_b[t] = rcp_approx((float)bsz);
     return K;
 }
 
@@ -490,9 +490,21 @@ __device__ __forceinline__ int optics_survival(const DetParams& dp, const PropPa
 // is a float, its reciprocal roots are of normal numbers.  100,000 segments of
 // bunch 5, 10 m slabs: 1.35 ms, with delta_at's layer selects in every slab
 // 3.70 ms.
+
+// Calls slab(j) for j = 0 .. ns - 1, j as a float.
+template <typename F>
+__device__ __forceinline__ void for_slabs(int ns, F&& slab) {
+    if (ns <= 1 << 24) {
+        const float end = (float)ns;
+        for (float j = 0.0f; j < end; j += 1.0f) slab(j);
+    } else {   // a float does not count past 2^24
+        for (int j = 0; j < ns; ++j) slab((float)j);
+    }
+}
+
 __device__ __noinline__ float4 snell_path(const AtmParams& ap, float dz, float cos0, float dh) {
     const int ns = max(1, (int)ceilf(dz / dh));
-    const float step = dz / (float)ns, nsf = (float)ns;
+    const float step = dz / (float)ns;
     const float d0 = delta_at(ap, dz - 0.5f * step);
     const float A0 = (1.0f + d0) * cos0;
     const float inv0 = 1.0f / A0;
@@ -500,7 +512,7 @@ __device__ __noinline__ float4 snell_path(const AtmParams& ap, float dz, float c
     float sR = 0.0f, sT = 0.0f, sX = 0.0f, sA = 0.0f;
     const bool trans = ap.transmission != 0;
     FallingDelta delta(ap);
-    for (float j = 0.0f; j < nsf; j += 1.0f) {
+    for_slabs(ns, [&](const float j) {
         const float h = dz - (j + 0.5f) * step;
         const float dj = delta.at(ap, h);
         const float D = (dj - d0) * (2.0f + dj + d0);
@@ -514,7 +526,7 @@ __device__ __noinline__ float4 snell_path(const AtmParams& ap, float dz, float c
             sX = fmaf(dj, g, sX);
             sA = fmaf(ex2_approx(ap.aer_c2 * h), g, sA);
         }
-    }
+    });
     return make_float4((1.0f + d0) * step * sR, fmaf(step, sT, dz * t0), ap.rho_per_delta * step * sX,
                        ap.aer_hobs * step * sA);
 }
@@ -544,9 +556,8 @@ __device__ __noinline__ float4 snell_path_sph(const AtmParams& ap, float dz, flo
     absolute = !line;
     float sPhi = 0.0f, sT = 0.0f, sX = 0.0f, sA = 0.0f;
     const bool trans = ap.transmission != 0;
-    const float nsf = (float)ns;
     FallingDelta delta(ap);
-    for (float j = 0.0f; j < nsf; j += 1.0f) {
+    for_slabs(ns, [&](const float j) {
         const float h = dz - (j + 0.5f) * step;
         const float dj = delta.at(ap, h);
         const float r_out = re - j * step, r_in = r_out - step;
@@ -565,7 +576,7 @@ __device__ __noinline__ float4 snell_path_sph(const AtmParams& ap, float dz, flo
             sX = fmaf(dj, t, sX);
             sA = fmaf(ex2_approx(ap.aer_c2 * h), t, sA);
         }
-    }
+    });
     return make_float4(ap.rg * sPhi, sT, ap.rho_per_delta * sX, ap.aer_hobs * sA);
 }
 
@@ -621,9 +632,8 @@ __device__ __noinline__ bool snell_path_cyl(const AtmParams& ap, float dz, float
     };
     bool reach = true;
     const bool trans = ap.transmission != 0;
-    const float nsf = (float)ns;
     FallingDelta delta(ap);
-    for (float j = 0.0f; j < nsf; j += 1.0f) {
+    for_slabs(ns, [&](const float j) {
         const float h = dz - (j + 0.5f) * step;
         const float dc = (refr || trans) ? delta.at(ap, h) : 0.0f;   // the shell's n - 1
         const float dj = refr ? dc : 0.0f;                                      // in the geometry
@@ -643,7 +653,7 @@ __device__ __noinline__ bool snell_path_cyl(const AtmParams& ap, float dz, float
             sX = fmaf(dc, s3, sX);
             sA = fmaf(ex2_approx(ap.aer_c2 * h), s3, sA);
         }
-    }
+    });
     out.chi = sChi + cChi;
     out.axial = sAx + cAx;
     out.ct = sCt + cCt;

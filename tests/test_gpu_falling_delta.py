@@ -33,3 +33,26 @@ def test_emission_at_layer_boundaries(dh, n_layers):
     o = oracle.propagate(segs, oracle.make_atm(oracle.ATM_LAYERED, layered=lay), hist=synth.histogram_400(),
                          tel=synth.grid_telescopes(), bunch=1, refraction=True, transmission=True, seed=5, snell_dh=dh)
     assert PU.compare(g, o, bunch=1)["matched"] > 500
+
+
+def test_more_slabs_than_a_float_counts():
+    """175 km of height in slabs of 1 cm: 1.7e7 slabs, more than 2^24.  In a
+    homogeneous medium no slab bends the path: the same ground points as with
+    thick slabs, bit for bit."""
+    pytest.importorskip("torch")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_2405_04229_gb300 import binding as B
+    from paper_2405_04229_gb300 import synth
+    segs = synth.shower_segments(2, 10.0, 0.0, 1e12, seed=3)
+    segs["z0"][:] = 175_000.0
+    segs["length"][:] = 1.0
+    segs["inv_gamma2"][:] = np.float32(1e-9)
+    atm = B.Atmosphere(kind=B.CS_ATM_HOMOGENEOUS, hom_delta=2.9e-4, refraction=True)
+    det = B.Detector(hist=synth.histogram_400())
+    assert (175_000.0 - 2000.0) / 0.01 > 2**24
+    a, b = (B.propagate_host(segs, atm, det, seed=5, bunch=20, records=True, snell_dh=dh) for dh in (0.01, 1000.0))
+    assert a["n_records"] == b["n_records"] > 0
+    ra, rb = (np.sort(r["records"], order=["seg", "k", "i"]) for r in (a, b))
+    for k in ("x", "y", "status"):
+        assert np.array_equal(ra[k], rb[k]), k
