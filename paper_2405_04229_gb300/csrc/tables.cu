@@ -89,7 +89,7 @@ __device__ inline double div_known(double x, double c, double rc) {
 }
 
 // Breakpoints of n(h) strictly inside (h_obs, h_e), between h_obs and h_e; returns their number.
-__device__ inline int piece_cuts(const AtmF64& a, double h_e, double* cuts) {
+__host__ __device__ inline int piece_cuts(const AtmF64& a, double h_e, double* cuts) {
     int nc = 0;
     cuts[nc++] = a.h_obs;
     if (a.kind == CS_ATM_LAYERED) {
@@ -152,12 +152,7 @@ struct PieceTable {
     const int* begin;
     const PiecePoint* pt;
 };
-__global__ void piece_count_kernel(AtmF64 a, int* begin) {
-    double cuts[kMaxNodes + 3];
-    const int nc = piece_cuts(a, 1e300, cuts);   // (the last piece is open)
-    begin[0] = 0;
-    for (int p = 0; p + 2 < nc; ++p) begin[p + 1] = begin[p] + kGL * (int)ceil((cuts[p + 1] - cuts[p]) / kSubMax);
-}
+constexpr int kPieceMax = 1 << 16;   // points tabulated; pieces beyond are formed where they are used
 __global__ void piece_points_kernel(AtmF64 a, const int* begin, PiecePoint* pt) {   // one block per piece
     double cuts[kMaxNodes + 3];
     const int nc = piece_cuts(a, 1e300, cuts), p = blockIdx.x;
@@ -213,15 +208,18 @@ __device__ void node_fields(const AtmF64& a, const PieceTable& tab, double h_e, 
             }
         }
     };
-    for (int p = 0; p + 2 < nc && p < tab.n; ++p) {
+    int p = 0;
+    for (; p + 2 < nc && p < tab.n; ++p) {
         const int end = __ldg(tab.begin + p + 1);
         for (int i = __ldg(tab.begin + p); i < end; ++i) {
             const PiecePoint* q = tab.pt + i;
             add(PiecePoint{__ldg(&q->h), __ldg(&q->wt), __ldg(&q->d), __ldg(&q->rho), __ldg(&q->ea)});
         }
     }
-    const Piece last(a, cuts[nc - 2], cuts[nc - 1]);
-    for (int i = 0; i < last.n; ++i) add(last.at(a, i));
+    for (; p + 1 < nc; ++p) {
+        const Piece piece(a, cuts[p], cuts[p + 1]);
+        for (int i = 0; i < piece.n; ++i) add(piece.at(a, i));
+    }
     if (a.spherical) {
         // G_R = (arc length correction on the ground sphere) cos^3 / sin, G_t = c dt cos,
         // G_X = X cos, G_A = A cos
@@ -587,25 +585,23 @@ extern "C" cs_status cs_atmosphere_create(const cs_atmosphere_desc* d, cs_atmosp
         (e = cudaMemcpy(drows, brows.data(), brows.size() * sizeof(int), cudaMemcpyHostToDevice)) != cudaSuccess)
         return fail("copy");
     // the points of the pieces between breakpoints (which all rows and labels share)
-    int n_cuts = 0;
     {
-        int begin[kMaxNodes + 3] = {0};
-        if (d->kind == CS_ATM_LAYERED) {
-            for (int k = 1; k < a.n_layers; ++k) n_cuts += a.lay_h[k] > a.h_obs;
-            n_cuts += a.h_top > a.h_obs;
-        } else if (d->kind == CS_ATM_LINEAR) {
-            n_cuts += a.lin_h1 > a.h_obs;
-        } else if (d->kind == CS_ATM_TABLE) {
-            for (int k = 1; k < a.n_nodes; ++k) n_cuts += a.node_h[k] > a.h_obs;
+        double cuts[kMaxNodes + 3];
+        const int nc = piece_cuts(a, 1e300, cuts);   // (the last piece is open)
+        std::vector<int> begin(1, 0);
+        for (int p = 0; p + 2 < nc; ++p) {
+            const double end = begin[p] + kGL * ceil((cuts[p + 1] - cuts[p]) / kSubMax);
+            if (!(end <= kPieceMax)) break;
+            begin.push_back((int)end);
         }
-        if ((e = cudaMalloc(&h->d_piece_begin, sizeof begin)) != cudaSuccess) return fail("pieces");
-        if (n_cuts) {
-            piece_count_kernel<<<1, 1>>>(a, h->d_piece_begin);
-            if ((e = cudaMemcpy(begin, h->d_piece_begin, sizeof begin, cudaMemcpyDeviceToHost)) != cudaSuccess) return fail("pieces");
-            if ((e = cudaMalloc(&h->d_pieces, begin[n_cuts] * sizeof(PiecePoint))) != cudaSuccess) return fail("pieces");
-            piece_points_kernel<<<n_cuts, 128>>>(a, h->d_piece_begin, (PiecePoint*)h->d_pieces);
+        h->n_pieces = (int)begin.size() - 1;
+        if (h->n_pieces) {
+            if ((e = cudaMalloc(&h->d_piece_begin, begin.size() * sizeof(int))) != cudaSuccess ||
+                (e = cudaMemcpy(h->d_piece_begin, begin.data(), begin.size() * sizeof(int), cudaMemcpyHostToDevice)) != cudaSuccess ||
+                (e = cudaMalloc(&h->d_pieces, begin.back() * sizeof(PiecePoint))) != cudaSuccess)
+                return fail("pieces");
+            piece_points_kernel<<<h->n_pieces, 128>>>(a, h->d_piece_begin, (PiecePoint*)h->d_pieces);
         }
-        h->n_pieces = n_cuts;
     }
     const PieceTable pieces = piece_table(h);
     const int T = 128;
