@@ -1346,10 +1346,15 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
             // rows and statuses of a round agree more often (measured 2-3 % faster), and with
             // the LV3 pre-filter whole rounds skip the correction (1.08x on the inclined
             // shower).  The draws stay keyed by the segments' own indices.
+            // The stepper's rounds last as long as their highest photon, so its segments are taken
+            // in order of height (100,000 segments of bunch 5: 1376 -> 1159 us), unless the LV3
+            // pre-filter is to skip whole rounds.
             int slot = lane;
             {
                 unsigned int word = ~0u;   // empty slots last
-                if (Kt0 > 0) {
+                if (TR && !pp.lv3) {
+                    if (Kt0 > 0) word = __float_as_uint(fmaxf(W.segB[lane].x, 0.0f));
+                } else if (Kt0 > 0) {
                     const float4 A = W.segA[lane], C = W.segC[lane];
                     float gx, gy;
                     if (SPH) {   // start point carried along P to the observation level
