@@ -30,9 +30,9 @@ namespace {
 constexpr int kThreads = 256;           // exact tracer: threads per block
 constexpr int kThreadsSur = 512;        // surrogate: four warpgroups per block
 constexpr int kMaxThreads = 512;
-constexpr int kTile = 256;              // segments per tile, one per thread (the first kTile threads)
+constexpr int kTile = 128;              // segments per tile, one per thread (the first kTile threads)
 constexpr int kSubCap = 512;            // sub-steps per round
-constexpr int kMapCap = 2048;           // bunches per window of the bunch -> sub-step map
+constexpr int kMapCap = 1024;           // bunches per window of the bunch -> sub-step map
 constexpr int kKShift = 8;              // sub-step record: segment (8 bits) | k << 8
 constexpr int kQBits = 10;              // map entry: sub-step (10 bits) | bunch index << 10
 
@@ -81,7 +81,13 @@ static_assert(4 * (kSmemPass + 1024) <= 228 * 1024, "four exact-tracer blocks pe
 
 // The surrogate instances keep the tensor-core network's buffers after the tile.
 constexpr size_t kTcSmemOffset = (sizeof(TileSmem) + 127) & ~(size_t)127;
+// Tiles of 128 segments, 512 sub-steps and 1,024 bunches, so that two blocks fit an SM: their warpgroups
+// wait for the tensor cores and at the block's barriers most of the time, and only other warps fill
+// that.  Two blocks of 64 registers a thread: 1e6 segments of bunch 5 946 us; one block with 256
+// segments, 2,048 bunches and 120 registers: 1169 us.  (One where the network splits its activations,
+// whose lo tiles take 64 KB more.)
 constexpr size_t smem_surrogate(bool split) { return kTcSmemOffset + TcSmem<kThreadsSur / 128>::bytes(split); }
+static_assert(2 * (smem_surrogate(false) + 1024) <= 228 * 1024, "two surrogate blocks per SM");
 
 // Exclusive block scan with one barrier; `buf` alternates between calls so a
 // scan never overwrites warp sums another warp may still be reading.
@@ -1794,8 +1800,8 @@ cs_status launch_kernel(unsigned grid, cudaStream_t stream, const PropParams& pp
     using f_ = std::false_type;
     const bool fl = pp.emission != 0, tr = pp.snell != 0;
     if (sur) {
-        if (ap.spherical) rec ? go_net(propagate_kernel<true, true, 1, true>) : go_net(propagate_kernel<true, true, 1, false>);
-        else rec ? go_net(propagate_kernel<true, false, 1, true>) : go_net(propagate_kernel<true, false, 1, false>);
+        if (ap.spherical) rec ? go_net(propagate_kernel<true, true, 2, true>) : go_net(propagate_kernel<true, true, 2, false>);
+        else rec ? go_net(propagate_kernel<true, false, 2, true>) : go_net(propagate_kernel<true, false, 2, false>);
     } else if (ap.spherical) {
         if (fl) tr ? exact(t_{}, t_{}, t_{}) : exact(t_{}, t_{}, f_{});
         else tr ? exact(t_{}, f_{}, t_{}) : exact(t_{}, f_{}, f_{});
@@ -1860,15 +1866,18 @@ cs_status set_smem_attributes() {
     CS_CUDA_TRY((set_exact_smem<true, false, true>(smem)));
     CS_CUDA_TRY((set_exact_smem<true, true, false>(smem)));
     CS_CUDA_TRY((set_exact_smem<true, true, true>(smem)));
-    CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, false, 1, false>, attr, smem_sur));
-    CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, false, 1, true>, attr, smem_sur));
-    CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, true, 1, false>, attr, smem_sur));
-    CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, true, 1, true>, attr, smem_sur));
+    CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, false, 2, false>, attr, smem_sur));
+    CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, false, 2, true>, attr, smem_sur));
+    CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, true, 2, false>, attr, smem_sur));
+    CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, true, 2, true>, attr, smem_sur));
     g_attr_done[dev] = true;
     return CS_OK;
 }
 
-int default_blocks_per_sm(const cs_opts& o) { return o.blocks_per_sm > 0 ? o.blocks_per_sm : (o.surrogate ? 1 : 4); }
+int default_blocks_per_sm(const cs_opts& o) {
+    if (o.blocks_per_sm > 0) return o.blocks_per_sm;
+    return !o.surrogate ? 4 : surrogate_view(o.surrogate)->split ? 1 : 2;   // what fits an SM
+}
 
 // How the launch deals n segments out: the grid of the persistent kernel and, for the exact
 // tracer, the segments of a warp tile and the parts that a tile's bunch rounds are split into.
