@@ -416,15 +416,45 @@ __global__ void transmission_kernel(const double2* __restrict__ hth, const doubl
 
 // The first-order baseline of each sample's fields, from the same FP32 table
 // and arithmetic as inference (so the network learns exactly what is added
-// back at inference).
-__global__ void baseline_kernel(SurrogateView sv, const double2* __restrict__ hth, const double* __restrict__ lam,
-                                size_t n, double h_obs, double* __restrict__ b3) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float3 b = surrogate_baseline(sv, (float)(hth[i].x - h_obs), (float)cos(hth[i].y), (float)(1.0 / (lam[i] * 1e9)));
-    b3[3 * i] = b.x;
-    b3[3 * i + 1] = b.y;
-    b3[3 * i + 2] = b.z;
+// back at inference), and the block's range of the first nt samples' targets
+// (fields less baseline): {lowest[3], highest[3]}.  On the device because the
+// labels would otherwise all travel to the host for it: 24 MB into pageable
+// memory and a logarithm each; the training below 29.7 -> 25.1 ms.
+constexpr int kBaseThreads = 256;
+__global__ void __launch_bounds__(kBaseThreads)
+baseline_kernel(SurrogateView sv, const double2* __restrict__ hth, const double* __restrict__ lam,
+                const Fields4* __restrict__ f, const double* __restrict__ Tphys, size_t n, size_t nt, double h_obs,
+                double* __restrict__ b3, double* __restrict__ range) {
+    __shared__ double red[kBaseThreads / 32][6];
+    const size_t i = (size_t)blockIdx.x * kBaseThreads + threadIdx.x;
+    double r[6] = {1e300, 1e300, 1e300, -1e300, -1e300, -1e300};
+    if (i < n) {
+        const float3 b = surrogate_baseline(sv, (float)(hth[i].x - h_obs), (float)cos(hth[i].y), (float)(1.0 / (lam[i] * 1e9)));
+        b3[3 * i] = b.x;
+        b3[3 * i + 1] = b.y;
+        b3[3 * i + 2] = b.z;
+        if (i < nt) {
+            const double y[3] = {f[i].x - b.x, f[i].y - b.y, log(Tphys[i]) - b.z};
+            for (int k = 0; k < 3; ++k) {   // (as with the host's comparisons, a NaN is passed over)
+                r[k] = fmin(r[k], y[k]);
+                r[3 + k] = fmax(r[3 + k], y[k]);
+            }
+        }
+    }
+    for (int k = 0; k < 6; ++k) {
+        for (int o = 16; o > 0; o >>= 1) {
+            const double v = __shfl_xor_sync(0xffffffffu, r[k], o);
+            r[k] = k < 3 ? fmin(r[k], v) : fmax(r[k], v);
+        }
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][k] = r[k];
+    }
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        const int k = threadIdx.x;
+        double v = red[0][k];
+        for (int w = 1; w < kBaseThreads / 32; ++w) v = k < 3 ? fmin(v, red[w][k]) : fmax(v, red[w][k]);
+        range[(size_t)blockIdx.x * 6 + k] = v;
+    }
 }
 
 // Normalised inputs (h_e - h_obs, cos(theta0), 1/lambda_nm) and targets: the
@@ -546,7 +576,8 @@ cs_status alloc(void** p, size_t bytes) {
 // Bound by latency: a row's three MMA round trips and 192 tanh leave little to
 // overlap within a warp, so what counts is warps per SM.  Two blocks of 512
 // threads (64 registers; one block where the split activations need their lo
-// tiles) instead of one of 256: 1e6 points EVAL_MS.
+// tiles) instead of one of 256: 1e6 points 153 -> 98 us, 90 us with layer 1 and the
+// biases as kernel parameters (SurrogateNet).
 constexpr int kEvalThreads = 512;
 template <bool SPLIT>
 __global__ void __launch_bounds__(kEvalThreads, SPLIT ? 1 : 2)
@@ -638,11 +669,24 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
     cudaStream_t s = nullptr;
     const size_t nt = (size_t)cfg.n_train, nh = (size_t)cfg.n_heldout, n_all = nt + nh;
     const int B = cfg.batch;
+    // buffers are cut from a few large allocations: each one of its own costs a mapping and, at the
+    // end, an unmapping
     std::vector<void*> bufs;
+    char* slab = nullptr;
+    size_t slab_left = 0;
     auto A = [&](size_t bytes) -> void* {
-        void* p = nullptr;
-        if (alloc(&p, bytes) != CS_OK) return nullptr;
-        bufs.push_back(p);
+        bytes = (bytes + 255) & ~(size_t)255;
+        if (bytes > slab_left) {
+            void* p = nullptr;
+            const size_t size = std::max<size_t>(bytes, (size_t)32 << 20);
+            if (alloc(&p, size) != CS_OK) return nullptr;
+            bufs.push_back(p);
+            slab = (char*)p;
+            slab_left = size;
+        }
+        void* p = slab;
+        slab += bytes;
+        slab_left -= bytes;
         return p;
     };
     auto cleanup = [&]() {
@@ -697,13 +741,6 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
                                                                    cfg.theta_max, atm->lambda_min, atm->lambda_max,
                                                                    hth, lam);
     if ((st = exact_fields(atm, hth, n_all, lab, s)) != CS_OK) { cleanup(); return st; }
-    std::vector<Fields4> hl(n_all);
-    cudaError_t e = cudaMemcpy(hl.data(), lab, n_all * sizeof(Fields4), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) { set_last_error("labels", e); cleanup(); return CS_ERR_CUDA; }
-    std::vector<double2> hhth(n_all);
-    std::vector<double> hlam(n_all);
-    cudaMemcpy(hhth.data(), hth, n_all * sizeof(double2), cudaMemcpyDeviceToHost);
-    cudaMemcpy(hlam.data(), lam, n_all * sizeof(double), cudaMemcpyDeviceToHost);
     // normalisation from the domain (inputs) and the training labels (outputs)
     Norm nm;
     const double il0 = 1.0 / (atm->lambda_max * 1e9), il1 = 1.0 / (atm->lambda_min * 1e9);
@@ -721,8 +758,6 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
     transmission_kernel<<<(unsigned)((n_all + 255) / 256), 256, 0, s>>>(
         hth, lam, lab, n_all, atm->rayl_X0, atm->rayl_lambda0, atm->aer_tau0 / atm->aer_H, atm->aer_lambda0,
         atm->aer_alpha, atm->p.transmission, Tphys);
-    std::vector<double> Tp(n_all);
-    cudaMemcpy(Tp.data(), Tphys, n_all * sizeof(double), cudaMemcpyDeviceToHost);
     // ---- the first-order baseline: FP64 vertical integrals on a fine grid of heights ----
     constexpr int kBaseN = 4096;
     SurrogateView bv;
@@ -753,16 +788,19 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
     }
     double* b3 = (double*)A(n_all * 3 * sizeof(double));
     if (!b3) { cudaFree(d_base); cleanup(); return CS_ERR_CUDA; }
-    baseline_kernel<<<(unsigned)((n_all + 255) / 256), 256, 0, s>>>(bv, hth, lam, n_all, atm->p.h_obs, b3);
-    std::vector<double> hb3(n_all * 3);
-    cudaMemcpy(hb3.data(), b3, n_all * 3 * sizeof(double), cudaMemcpyDeviceToHost);
+    const unsigned base_blocks = (unsigned)((n_all + kBaseThreads - 1) / kBaseThreads);
+    double* d_range = (double*)A((size_t)base_blocks * 6 * sizeof(double));
+    if (!d_range) { cudaFree(d_base); cleanup(); return CS_ERR_CUDA; }
+    baseline_kernel<<<base_blocks, kBaseThreads, 0, s>>>(bv, hth, lam, lab, Tphys, n_all, nt, atm->p.h_obs, b3, d_range);
     // output normalisation from the training targets (fields less baseline)
+    std::vector<double> range((size_t)base_blocks * 6);
+    cudaError_t e = cudaMemcpy(range.data(), d_range, range.size() * sizeof(double), cudaMemcpyDeviceToHost);
+    if (e != cudaSuccess) { set_last_error("labels", e); cudaFree(d_base); cleanup(); return CS_ERR_CUDA; }
     double mn[3] = {1e300, 1e300, 1e300}, mx[3] = {-1e300, -1e300, -1e300};
-    for (size_t i = 0; i < nt; ++i) {
-        const double r[3] = {hl[i].x - hb3[3 * i], hl[i].y - hb3[3 * i + 1], log(Tp[i]) - hb3[3 * i + 2]};
+    for (size_t b = 0; b < base_blocks; ++b) {
         for (int k = 0; k < 3; ++k) {
-            mn[k] = std::min(mn[k], r[k]);
-            mx[k] = std::max(mx[k], r[k]);
+            mn[k] = std::min(mn[k], range[6 * b + k]);
+            mx[k] = std::max(mx[k], range[6 * b + 3 + k]);
         }
     }
     for (int k = 0; k < 3; ++k) {
@@ -942,10 +980,17 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
     sg->lambda_min = atm->lambda_min;
     sg->lambda_max = atm->lambda_max;
     // ---- held-out errors in physical units, through the inference path ------------
+    std::vector<Fields4> hl(nh);
+    std::vector<double2> hhth(nh);
+    std::vector<double> hlam(nh), Tp(nh);
+    cudaMemcpy(hl.data(), lab + nt, nh * sizeof(Fields4), cudaMemcpyDeviceToHost);
+    cudaMemcpy(hhth.data(), hth + nt, nh * sizeof(double2), cudaMemcpyDeviceToHost);
+    cudaMemcpy(hlam.data(), lam + nt, nh * sizeof(double), cudaMemcpyDeviceToHost);
+    cudaMemcpy(Tp.data(), Tphys + nt, nh * sizeof(double), cudaMemcpyDeviceToHost);
     std::vector<float4> hin(nh);
     for (size_t i = 0; i < nh; ++i) {
-        const double2 a = hhth[nt + i];
-        hin[i] = make_float4((float)(a.x - atm->p.h_obs), (float)cos(a.y), (float)(1.0 / (hlam[nt + i] * 1e9)), 0.f);
+        const double2 a = hhth[i];
+        hin[i] = make_float4((float)(a.x - atm->p.h_obs), (float)cos(a.y), (float)(1.0 / (hlam[i] * 1e9)), 0.f);
     }
     float4 *din = (float4*)A(nh * sizeof(float4)), *dout = (float4*)A(nh * sizeof(float4));
     std::vector<float4> hout(nh);
@@ -961,17 +1006,18 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
     }
     std::vector<double> er[3];
     for (size_t i = 0; i < nh; ++i) {
-        const double th = hhth[nt + i].y, c = cos(th), sn = sin(th);
-        er[0].push_back(fabs(hout[i].x - hl[nt + i].x) * sn / (c * c * c));   // displacement [m]
-        er[1].push_back(fabs(hout[i].y - hl[nt + i].y) / (c * kC));          // delay [s]
-        er[2].push_back(fabs(hout[i].z - Tp[nt + i]));                        // transmission
+        const double th = hhth[i].y, c = cos(th), sn = sin(th);
+        er[0].push_back(fabs(hout[i].x - hl[i].x) * sn / (c * c * c));   // displacement [m]
+        er[1].push_back(fabs(hout[i].y - hl[i].y) / (c * kC));          // delay [s]
+        er[2].push_back(fabs(hout[i].z - Tp[i]));                        // transmission
     }
     cs_surrogate_stats& S = sg->stats;
     memset(&S, 0, sizeof S);
     for (int k = 0; k < 3; ++k) {
-        std::sort(er[k].begin(), er[k].end());
-        S.heldout_p99[k] = er[k][(size_t)(0.99 * (er[k].size() - 1))];
-        S.heldout_max[k] = er[k].back();
+        const auto p99 = er[k].begin() + (size_t)(0.99 * (er[k].size() - 1));
+        std::nth_element(er[k].begin(), p99, er[k].end());   // (what lies above it comes after it)
+        S.heldout_p99[k] = *p99;
+        S.heldout_max[k] = *std::max_element(p99, er[k].end());
     }
     S.final_loss = last_loss;
     S.steps = total;
