@@ -738,14 +738,15 @@ enum { kModeMain = 0, kModeCheck = 1, kModeExact = 2 };
 // FIX: the launch configuration as compile-time constants instead of parameter tests, whose uniform
 // branches cost issue slots.  kFixed, kFixedOptics: refraction, transmission and tables on,
 // histogram, telescopes and time sums on, without and with camera optics (the LV3 switch stays a
-// test); kAny: tested.  1e6 segments: optics 252 -> 233 us, fluorescence 177 -> 168 us.
+// test; the network with single activations); kAny: tested.  1e6 segments: optics 252 -> 233 us,
+// fluorescence 177 -> 168 us, the network 946 -> 847 us (its two forms in one instance spilled).
 enum { kAny = 0, kFixed = 1, kFixedOptics = 2 };
 template <bool SURR, bool SPH, bool REC, bool FL, bool TR, int MODE = kModeMain, int FIX = kAny, typename SM>
 __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, long long base,
                                       const PropParams& pp, const AtmParams& ap, const DetParams& dp,
                                       const OutParams& op, const NetParam<SURR>& sv, TcSmem<kThreadsSur / 128>* tcs,
                                       Tally& T) {
-    static_assert(!(FIX && (SURR || TR || MODE != kModeMain)), "the fixed configurations are the table tracer's");
+    static_assert(!(FIX && (TR || MODE != kModeMain)), "the fixed configurations are the tables' and the network's");
     const bool c_refr = FIX || ap.refraction, c_trans = FIX || ap.transmission, c_tables = FIX || ap.use_tables;
     const bool c_lv3 = pp.lv3 != 0, c_cam = FIX == kFixedOptics || (!FIX && dp.cam_n > 0), c_hist = FIX || dp.nx > 0;
     const bool c_tel = FIX || dp.n_tel > 0, c_time = FIX || op.tel_time != nullptr;
@@ -831,7 +832,7 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                             use_net ? fmaf(sv.in_scale[1], cos_z, sv.in_shift[1]) : 0.0f,
                             use_net ? fmaf(sv.in_scale[2], inv_l, sv.in_shift[2]) : 0.0f};
         float y[3];
-        const bool ok = sv.split ? net128_tc<true>(sv, *tcs, x, y) : net128_tc<false>(sv, *tcs, x, y);
+        const bool ok = !FIX && sv.split ? net128_tc<true>(sv, *tcs, x, y) : net128_tc<false>(sv, *tcs, x, y);
         use_net = use_net && ok;   // a tensor-core wait that gave up: the tables take over
         if (use_net) {   // the network's part plus the first-order baseline
             const float3 bl = surrogate_baseline(sv, dz, cos_z, inv_l);
@@ -1642,7 +1643,7 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                         const bool active = p < wn;
                         const unsigned int e = S.map[active ? p : pw];
                         const int qs = (int)(e & ((1u << kQBits) - 1));
-                        if (bunch<SURR, SPH, REC, FL, TR>(S, qs, (int)(e >> kQBits), active, base, pp, ap, dp, op, sv,
+                        if (bunch<SURR, SPH, REC, FL, TR, kModeMain, FIX>(S, qs, (int)(e >> kQBits), active, base, pp, ap, dp, op, sv,
                                                           tcs, T)) {   // left to the exact pass: mark its warp tile
                             const int sg = __float_as_int(S.sub[qs].w) & ((1 << kKShift) - 1);
                             mark_group(scratch, (pp.n + kWTile - 1) / kWTile, pp.tiles_per_bit,
@@ -1800,8 +1801,12 @@ cs_status launch_kernel(unsigned grid, cudaStream_t stream, const PropParams& pp
     using f_ = std::false_type;
     const bool fl = pp.emission != 0, tr = pp.snell != 0;
     if (sur) {
-        if (ap.spherical) rec ? go_net(propagate_kernel<true, true, 2, true>) : go_net(propagate_kernel<true, true, 2, false>);
-        else rec ? go_net(propagate_kernel<true, false, 2, true>) : go_net(propagate_kernel<true, false, 2, false>);
+        auto network = [&](auto sph) {
+            constexpr bool S = decltype(sph)::value;
+            if (fix && !cam && !rec && !net.split) go_net(propagate_kernel<true, S, 2, false, false, false, false, kFixed>);
+            else rec ? go_net(propagate_kernel<true, S, 2, true>) : go_net(propagate_kernel<true, S, 2, false>);
+        };
+        ap.spherical ? network(t_{}) : network(f_{});
     } else if (ap.spherical) {
         if (fl) tr ? exact(t_{}, t_{}, t_{}) : exact(t_{}, t_{}, f_{});
         else tr ? exact(t_{}, f_{}, t_{}) : exact(t_{}, f_{}, f_{});
@@ -1867,6 +1872,8 @@ cs_status set_smem_attributes() {
     CS_CUDA_TRY((set_exact_smem<true, true, false>(smem)));
     CS_CUDA_TRY((set_exact_smem<true, true, true>(smem)));
     CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, false, 2, false>, attr, smem_sur));
+    CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, false, 2, false, false, false, false, kFixed>, attr, smem_sur));
+    CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, true, 2, false, false, false, false, kFixed>, attr, smem_sur));
     CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, false, 2, true>, attr, smem_sur));
     CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, true, 2, false>, attr, smem_sur));
     CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, true, 2, true>, attr, smem_sur));
