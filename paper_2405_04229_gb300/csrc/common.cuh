@@ -201,7 +201,9 @@ struct __align__(16) Fields4 {   // {G_R, G_t, G_X, G_A} in FP64
     double x, y, z, w;
 };
 // Exact FP64 {G_R, G_t, G_X, G_A} at samples {h_e [m], theta0 [rad]} (device arrays).
-cs_status exact_fields(const cs_atmosphere* atm, const double2* d_in, size_t n, Fields4* d_out, cudaStream_t stream);
+// scratch: exact_fields_scratch(n) bytes of device memory
+size_t exact_fields_scratch(size_t n);
+cs_status exact_fields(const cs_atmosphere* atm, const double2* d_in, size_t n, Fields4* d_out, void* scratch, cudaStream_t stream);
 // FP64 vertical integrals from h_obs up to each height h [m] (device arrays):
 // {int (n - 1) dh, n(h) - 1, int 100 rho dh [g/cm^2], int exp(-h / H_A) dh}.
 cs_status column_fields(const cs_atmosphere* atm, const double* d_h, size_t n, Fields4* d_out, cudaStream_t stream);

@@ -740,7 +740,9 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
     sample_kernel<<<(unsigned)((n_all + 255) / 256), 256, 0, s>>>(k0, k1, 1u, n_all, cfg.h_min, cfg.h_max, bands,
                                                                    cfg.theta_max, atm->lambda_min, atm->lambda_max,
                                                                    hth, lam);
-    if ((st = exact_fields(atm, hth, n_all, lab, s)) != CS_OK) { cleanup(); return st; }
+    void* label_scratch = A(exact_fields_scratch(n_all));
+    if (!label_scratch) { cleanup(); return CS_ERR_CUDA; }
+    if ((st = exact_fields(atm, hth, n_all, lab, label_scratch, s)) != CS_OK) { cleanup(); return st; }
     // normalisation from the domain (inputs) and the training labels (outputs)
     Norm nm;
     const double il0 = 1.0 / (atm->lambda_max * 1e9), il1 = 1.0 / (atm->lambda_min * 1e9);

@@ -328,10 +328,51 @@ __global__ void column_kernel(AtmF64 a, const double* h_in, size_t n, Fields4* o
     out[i] = Fields4{sI, de, sX, sA};
 }
 
-// One thread per sample: the exact FP64 fields at (h_e, theta0).
-__global__ void exact_fields_kernel(AtmF64 a, PieceTable tab, const double2* in, size_t n, Fields4* out) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+// Samples by height, the highest first: a sample's integral has as many points as its height gives
+// it, and a warp takes as long as its longest.  Bins of 250 m by counting; the order within a bin is
+// arbitrary (each sample is integrated by itself).
+constexpr int kHeightBins = 256, kOrderThreads = 256;
+__device__ __forceinline__ int height_bin(const AtmF64& a, double h) {
+    return kHeightBins - 1 - (int)fmin(fmax((h - a.h_obs) * (1.0 / 250.0), 0.0), (double)(kHeightBins - 1));
+}
+__global__ void __launch_bounds__(kOrderThreads) bin_count_kernel(AtmF64 a, const double2* in, unsigned int n, unsigned int* count) {
+    __shared__ unsigned int c[kHeightBins];
+    c[threadIdx.x] = 0u;
+    __syncthreads();
+    for (unsigned int i = blockIdx.x * kOrderThreads + threadIdx.x; i < n; i += gridDim.x * kOrderThreads)
+        atomicAdd(c + height_bin(a, in[i].x), 1u);
+    __syncthreads();
+    if (c[threadIdx.x]) atomicAdd(count + threadIdx.x, c[threadIdx.x]);
+}
+__global__ void __launch_bounds__(kOrderThreads)
+bin_scatter_kernel(AtmF64 a, const double2* in, unsigned int n, const unsigned int* count, unsigned int* taken, unsigned int* order) {
+    __shared__ unsigned int first[kHeightBins];
+    const int t = threadIdx.x;
+    unsigned int v = count[t];
+    first[t] = v;
+    __syncthreads();
+    for (int o = 1; o < kHeightBins; o <<= 1) {
+        const unsigned int w = t >= o ? first[t - o] : 0u;
+        __syncthreads();
+        first[t] += w;
+        __syncthreads();
+    }
+    first[t] -= v;
+    __syncthreads();
+    const unsigned int i = blockIdx.x * kOrderThreads + t;
+    if (i < n) {
+        const int b = height_bin(a, in[i].x);
+        order[first[b] + atomicAdd(taken + b, 1u)] = i;
+    }
+}
+static_assert(kHeightBins == kOrderThreads, "one bin per thread");
+
+// One thread per sample, in the order given: the exact FP64 fields at (h_e, theta0).  In the samples'
+// own order 17 of 32 lanes worked, 278,528 samples 10.0 ms; by height about 5 ms (training with these labels 25.1 -> 20.3 ms).
+__global__ void exact_fields_kernel(AtmF64 a, PieceTable tab, const double2* in, const unsigned int* order, size_t n, Fields4* out) {
+    const size_t j = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    const size_t i = order[j];
     const double h_e = in[i].x, th = in[i].y;
     const double cos0 = cos(th), sin0 = sin(th);
     double f[4];
@@ -639,10 +680,18 @@ cs_status column_fields(const cs_atmosphere* atm, const double* d_h, size_t n, F
     return CS_OK;
 }
 
-cs_status exact_fields(const cs_atmosphere* atm, const double2* d_in, size_t n, Fields4* d_out, cudaStream_t stream) {
+size_t exact_fields_scratch(size_t n) { return (2 * kHeightBins + n) * sizeof(unsigned int); }
+
+cs_status exact_fields(const cs_atmosphere* atm, const double2* d_in, size_t n, Fields4* d_out, void* scratch, cudaStream_t stream) {
     if (n == 0) return CS_OK;
+    if (n > 0xFFFFFFFFu) return CS_ERR_INVALID_ARG;
+    unsigned int *count = (unsigned int*)scratch, *taken = count + kHeightBins, *order = taken + kHeightBins;
+    const unsigned int blocks = (unsigned int)((n + kOrderThreads - 1) / kOrderThreads);
+    CS_CUDA_TRY(cudaMemsetAsync(count, 0, 2 * kHeightBins * sizeof(unsigned int), stream));
+    bin_count_kernel<<<blocks < 608 ? blocks : 608, kOrderThreads, 0, stream>>>(atm->f64, d_in, (unsigned int)n, count);
+    bin_scatter_kernel<<<blocks, kOrderThreads, 0, stream>>>(atm->f64, d_in, (unsigned int)n, count, taken, order);
     exact_fields_kernel<<<(unsigned)((n + 127) / 128), 128, 0, stream>>>(
-        atm->f64, piece_table(atm), d_in, n, d_out);
+        atm->f64, piece_table(atm), d_in, order, n, d_out);
     CS_CUDA_TRY(cudaGetLastError());
     return CS_OK;
 }
