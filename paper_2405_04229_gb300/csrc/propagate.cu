@@ -1539,38 +1539,68 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                 process_tile(base, (int)std::min<long long>(pp.tile_segs, pp.n - base), part, 1 << pp.parts_log2);
             }
         } else {
-            // the exact pass takes the queued bunches 32 at a time, then the marked groups
-            // from their list (the cursor runs over both)
+            // the exact pass takes the queued bunches a block's worth at a time, then the marked groups
+            // from their list.  A bunch is integrated over as many sub-intervals as its height gives it
+            // and a warp takes as long as its longest: the block orders its entries by height, in bins
+            // of 1 km.  (In the queue's order 20 of 32 lanes
+            // worked; fluorescence on 1e6 segments 168 -> 158 us.)
             const unsigned int n_listed = __ldcg(scratch + 2);
-            const unsigned int n_q = min(__ldcg(scratch + 3), pp.q_cap), n_qc = (n_q + 31) / 32;
+            const unsigned int n_q = min(__ldcg(scratch + 3), pp.q_cap);
             const unsigned int* bits = scratch + kScratchCounters;
             const unsigned int* list = bits + (scratch_groups(n_wtiles, pp.tiles_per_bit) + 31) / 32;
+            struct Ordered {   // (over the warps' buffers, which hold nothing between units)
+                int first[64];
+                uint4 entry[NT];
+            };
+            static_assert(sizeof(Ordered) <= (NT / 32) * sizeof(WarpBuf), "fits the warps' buffers");
+            Ordered& O = *reinterpret_cast<Ordered*>(smem_raw);
+            for (unsigned int q0 = blockIdx.x * NT; q0 < n_q; q0 += gridDim.x * NT) {
+                uint4 ent = make_uint4(0u, 0u, 0xFFFFFFFFu, 0u);   // {segment, segment, sub-step (or none), bunch}
+                int bin = 63;
+                if (q0 + t < n_q) {
+                    const uint4 e = __ldcg(reinterpret_cast<const uint4*>(scratch + pp.q_off) + (q0 + t));
+                    const long long li = (long long)(((unsigned long long)e.y << 32) | e.x);
+                    const unsigned long long g = (unsigned long long)(li / kWTile) / (unsigned long long)pp.tiles_per_bit;
+                    if (!((__ldcg(bits + (g >> 5)) >> (g & 31)) & 1u)) {   // a tile the queue overflowed on is the group pass's
+                        ent = e;
+                        bin = 62 - (int)fminf(fmaxf((float)(pp.segs[li].z0 - ap.h_obs) * 1e-3f, 0.0f), 62.0f);
+                    }
+                }
+                __syncthreads();   // the warps are done with the unit before
+                if (t < 64) O.first[t] = 0;
+                __syncthreads();
+                const int at = atomicAdd(O.first + bin, 1);
+                __syncthreads();
+                if (t < 32) {   // counts to first places
+                    const int c0 = O.first[2 * t], c1 = O.first[2 * t + 1];
+                    int incl = c0 + c1;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+                        if (t >= o) incl += y;
+                    }
+                    O.first[2 * t] = incl - c0 - c1;
+                    O.first[2 * t + 1] = incl - c1;
+                }
+                __syncthreads();
+                O.entry[O.first[bin] + at] = ent;
+                __syncthreads();
+                ent = O.entry[t];
+                __syncthreads();
+                // lane j: its entry's segment in slot j, its sub-step in slot j
+                if (ent.z != 0xFFFFFFFFu) {
+                    const long long li = (long long)(((unsigned long long)ent.y << 32) | ent.x);
+                    const long long base_l = li - lane;   // so that base + slot is the segment's index
+                    import_segment<SPH, FL>(W, lane, pp.segs + li, pp, ap, dp, invalid, dropped, false);
+                    substep<SPH, FL>(W, W.sub[lane], lane, (int)ent.z, base_l, pp, ap);
+                    bunch<false, SPH, REC, FL, TR, kModeExact>(W, lane, (int)ent.w, true, base_l, pp, ap, dp, op, sv, tcs, T);
+                }
+            }
+            __syncwarp();
             for (;;) {
                 unsigned int idx = 0;
                 if (lane == 0) idx = atomicAdd(tile_ctr, 1u);
                 idx = __shfl_sync(0xffffffffu, idx, 0);
-                if (idx < n_qc) {
-                    // lane j: queue entry 32 idx + j, its segment in slot j, its sub-step in slot j
-                    const unsigned int qe = idx * 32u + (unsigned int)lane;
-                    bool act = qe < n_q;
-                    uint4 ent = make_uint4(0u, 0u, 0u, 0u);
-                    if (act) ent = __ldcg(reinterpret_cast<const uint4*>(scratch + pp.q_off) + qe);
-                    const long long li = (long long)(((unsigned long long)ent.y << 32) | ent.x);
-                    if (act) {   // a tile the queue overflowed on is the group pass's
-                        const unsigned long long g = (unsigned long long)(li / kWTile) / (unsigned long long)pp.tiles_per_bit;
-                        if ((__ldcg(bits + (g >> 5)) >> (g & 31)) & 1u) act = false;
-                    }
-                    const long long base_l = li - lane;   // so that base + slot is the segment's index
-                    if (act) {
-                        import_segment<SPH, FL>(W, lane, pp.segs + li, pp, ap, dp, invalid, dropped, false);
-                        substep<SPH, FL>(W, W.sub[lane], lane, (int)ent.z, base_l, pp, ap);
-                        bunch<false, SPH, REC, FL, TR, kModeExact>(W, lane, (int)ent.w, true, base_l, pp, ap, dp, op, sv,
-                                                                   tcs, T);
-                    }
-                    __syncwarp();
-                    continue;
-                }
-                idx -= n_qc;
                 if (idx >= n_listed) break;
                 const long long g = (long long)__ldcg(list + idx);
                 const long long t_end = std::min<long long>((g + 1) * pp.tiles_per_bit, n_wtiles);
