@@ -32,7 +32,7 @@ constexpr int kThreadsSur = 512;        // surrogate: four warpgroups per block
 constexpr int kMaxThreads = 512;
 constexpr int kTile = 128;              // segments per tile, one per thread (the first kTile threads)
 constexpr int kSubCap = 512;            // sub-steps per round
-constexpr int kMapCap = 1024;           // bunches per window of the bunch -> sub-step map
+constexpr int kMapCap = 1792;           // bunches per window of the bunch -> sub-step map
 constexpr int kKShift = 8;              // sub-step record: segment (8 bits) | k << 8
 constexpr int kQBits = 10;              // map entry: sub-step (10 bits) | bunch index << 10
 
@@ -81,11 +81,12 @@ static_assert(4 * (kSmemPass + 1024) <= 228 * 1024, "four exact-tracer blocks pe
 
 // The surrogate instances keep the tensor-core network's buffers after the tile.
 constexpr size_t kTcSmemOffset = (sizeof(TileSmem) + 127) & ~(size_t)127;
-// Tiles of 128 segments, 512 sub-steps and 1,024 bunches, so that two blocks fit an SM: their warpgroups
+// Tiles of 128 segments, 512 sub-steps and 1,792 bunches, so that two blocks fit an SM: their warpgroups
 // wait for the tensor cores and at the block's barriers most of the time, and only other warps fill
 // that.  Two blocks of 64 registers a thread: 1e6 segments of bunch 5 946 us; one block with 256
-// segments, 2,048 bunches and 120 registers: 1169 us.  (One where the network splits its activations,
-// whose lo tiles take 64 KB more.)
+// segments, 2,048 bunches and 120 registers: 1169 us.  A tile has about 1,250 bunches at bunch 5: in
+// windows of 1,024 a second, mostly empty one followed (847 us, so 829 us).  (One block where the
+// network splits its activations, whose lo tiles take 64 KB more.)
 constexpr size_t smem_surrogate(bool split) { return kTcSmemOffset + TcSmem<kThreadsSur / 128>::bytes(split); }
 static_assert(2 * (smem_surrogate(false) + 1024) <= 228 * 1024, "two surrogate blocks per SM");
 
