@@ -494,9 +494,10 @@ __device__ __forceinline__ int optics_survival(const DetParams& dp, const PropPa
 // The steppers are bound by issue slots (a slab is a chain of four special
 // functions; ~30 warps per SM hide it), so a slab's instructions are what
 // counts: its layer is kept and only left downwards (FallingDelta), its index
-// is a float, its reciprocal roots are of normal numbers.  100,000 segments of
-// bunch 5, 10 m slabs: 1.35 ms, with delta_at's layer selects in every slab
-// 3.70 ms.
+// is a float, its reciprocal roots are of normal numbers, and the plane's form
+// takes two slabs per packed FP32 instruction.  100,000 segments of bunch 5,
+// 10 m slabs: 3.70 ms with delta_at's layer selects in every slab, 1.38 ms with
+// the kept layer, 1.16 ms with rounds of like heights, 0.74 ms in pairs.
 
 // Calls slab(j) for j = 0 .. ns - 1, j as a float.
 template <typename F>
@@ -519,7 +520,7 @@ __device__ __noinline__ float4 snell_path(const AtmParams& ap, float dz, float c
     float sR = 0.0f, sT = 0.0f, sX = 0.0f, sA = 0.0f;
     const bool trans = ap.transmission != 0;
     FallingDelta delta(ap);
-    for_slabs(ns, [&](const float j) {
+    auto slab = [&](const float j) {
         const float h = dz - (j + 0.5f) * step;
         const float dj = delta.at(ap, h);
         const float D = (dj - d0) * (2.0f + dj + d0);
@@ -533,7 +534,43 @@ __device__ __noinline__ float4 snell_path(const AtmParams& ap, float dz, float c
             sX = fmaf(dj, g, sX);
             sA = fmaf(ex2_approx(ap.aer_c2 * h), g, sA);
         }
-    });
+    };
+    if (ns > 1 << 22) {
+        for_slabs(ns, slab);
+    } else {
+        // two slabs at a time in packed FP32 instructions, each in the operations and order of `slab`
+        auto two = [](float v) { return make_float2(v, v); };
+        const bool layered = ap.kind == CS_ATM_LAYERED;
+        const float nsf = (float)ns;
+        float2 j = make_float2(0.5f, 1.5f);   // index + 1/2
+        for (; j.x < nsf - 1.0f; j = __fadd2_rn(j, two(2.0f))) {
+            const float2 h = __ffma2_rn(make_float2(-j.x, -j.y), two(step), two(dz));
+            float2 d;
+            if (layered && !(h.y < delta.lo)) {
+                const float2 e = __fmul2_rn(two(delta.c2), h);
+                d = __fmul2_rn(two(delta.D), make_float2(ex2_approx(e.x), ex2_approx(e.y)));
+            } else {
+                d.x = delta.at(ap, h.x);
+                d.y = delta.at(ap, h.y);
+            }
+            const float2 D = __fmul2_rn(__fadd2_rn(d, two(-d0)), __fadd2_rn(__fadd2_rn(two(2.0f), d), two(d0)));
+            float2 Aj2 = __ffma2_rn(two(A0), two(A0), D);
+            Aj2 = make_float2(fmaxf(Aj2.x, 1e-12f), fmaxf(Aj2.y, 1e-12f));
+            const float2 inv = make_float2(rsqrt_approx(Aj2.x), rsqrt_approx(Aj2.y));
+            const float2 sum = __ffma2_rn(Aj2, inv, two(A0)), n = __fadd2_rn(two(1.0f), d), g = __fmul2_rn(n, inv);
+            const float2 w = __fmul2_rn(__fmul2_rn(D, inv), two(inv0)), t = __ffma2_rn(n, g, two(-t0));
+            sR = fmaf(-w.x, rcp_approx(sum.x), sR);
+            sR = fmaf(-w.y, rcp_approx(sum.y), sR);
+            sT = sT + t.x;
+            sT = sT + t.y;
+            if (trans) {
+                const float2 e = __fmul2_rn(two(ap.aer_c2), h);
+                sX = fmaf(d.y, g.y, fmaf(d.x, g.x, sX));
+                sA = fmaf(ex2_approx(e.y), g.y, fmaf(ex2_approx(e.x), g.x, sA));
+            }
+        }
+        if (j.x < nsf) slab(j.x - 0.5f);
+    }
     return make_float4((1.0f + d0) * step * sR, fmaf(step, sT, dz * t0), ap.rho_per_delta * step * sX,
                        ap.aer_hobs * step * sA);
 }
