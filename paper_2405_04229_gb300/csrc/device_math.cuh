@@ -52,6 +52,10 @@ __device__ __forceinline__ uint4 philox_rk(uint32_t c0, uint32_t c1, uint32_t c2
 // 24-bit uniform in [0, 1), exact in FP32 and FP64
 __device__ __forceinline__ float uniform24(uint32_t x) { return __uint2float_rn(x >> 8) * 0x1p-24f; }
 
+// packed FP32 operands
+__device__ __forceinline__ float2 two(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
+
 // ---- float-float (error-free transformations) ------------------------------
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     s = a + b;

@@ -123,8 +123,11 @@ static __global__ void gl_points_kernel(const AtmParams ap, float4* nodes, float
         const PieceLaw law = piece_law(ap, mid);
         const float y = (g < 8) ? fmaf(-half, gx, mid) : fmaf(half, gx, mid);
         const float d = piece_delta<false>(law, y), n = 1.0f + d;
-        nodes[k * 16 + g] = make_float4(half * c_gl16_w[g & 7], d, ap.rho_per_delta * d * n,
-                                        ap.aer_hobs * ex2_approx(ap.aer_c2 * y) * n);
+        float* at = reinterpret_cast<float*>(nodes + k * 16 + (g & ~1)) + (g & 1);   // points in pairs
+        at[0] = half * c_gl16_w[g & 7];
+        at[2] = d;
+        at[4] = ap.rho_per_delta * d * n;
+        at[6] = ap.aer_hobs * ex2_approx(ap.aer_c2 * y) * n;
         if (g == 0) ends[k] = xb;
         xa = xb;
     }
@@ -155,6 +158,26 @@ static __device__ __noinline__ float4 exact_fields_planar(const AtmParams* __res
         if (!reaches) return make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     }
     float aR = 0.0f, aT = 0.0f, aX = 0.0f, aA = 0.0f;
+    // Two points at a time in packed FP32 instructions (the sums in the points' order): X and A are
+    // the columns' integrands times q.  Fluorescence on 1e6 segments 158 -> 147 us.
+    auto add = [&](float2 wt, float2 d, float2 n, float2 X, float2 A) {
+        const float2 n2 = __fmul2_rn(n, n);
+        const float2 D = __fmul2_rn(__fadd2_rn(d, two(-de)), __fadd2_rn(__fadd2_rn(two(2.0f), d), two(de)));
+        const float2 f = __ffma2_rn(two(ne * ne), two(c2), D), q2 = make_float2(fmaxf(f.x, 1e-30f), fmaxf(f.y, 1e-30f));
+        const float2 iq = make_float2(rsqrt_approx(q2.x), rsqrt_approx(q2.y)), q = __fmul2_rn(q2, iq);
+        const float2 sR = __ffma2_rn(two(ne), two(c0), q), sT = __ffma2_rn(n2, two(c0), q);
+        const float2 vR = __fmul2_rn(__fmul2_rn(D, iq), make_float2(rcp_approx(sR.x), rcp_approx(sR.y)));
+        const float2 e = __fadd2_rn(__ffma2_rn(d, d, __fmul2_rn(two(2.0f), d)), two(-de));
+        const float2 t = __ffma2_rn(__fmul2_rn(two(c2), e), __fadd2_rn(n2, two(ne)), make_float2(-D.x, -D.y));
+        const float2 vT = __fmul2_rn(__fmul2_rn(t, iq), make_float2(rcp_approx(sT.x), rcp_approx(sT.y)));
+        aR = fmaf(wt.y, -vR.y, fmaf(wt.x, -vR.x, aR));
+        aT = fmaf(wt.y, vT.y, fmaf(wt.x, vT.x, aT));
+        if (trans) {
+            const float2 vX = __fmul2_rn(X, iq), vA = __fmul2_rn(A, iq);
+            aX = fmaf(wt.y, vX.y, fmaf(wt.x, vX.x, aX));
+            aA = fmaf(wt.y, vA.y, fmaf(wt.x, vA.x, aA));
+        }
+    };
     float x0 = 0.0f;
     // (2 km sub-intervals: the photon is not emitted above 256 km)
     const int n_gl = dz <= 256000.0f ? ap.n_gl : 0;
@@ -163,17 +186,10 @@ static __device__ __noinline__ float4 exact_fields_planar(const AtmParams* __res
         if (!(xb <= dz - 2000.0f)) break;
         const float4* p = ap.gl_nodes + k * 16;
 #pragma unroll
-        for (int g = 0; g < 16; ++g) {
-            const float4 v = __ldg(p + g);
-            const float wt = v.x, d = v.y;
-            const float n = 1.0f + d, n2 = n * n;
-            const float D = (d - de) * (2.0f + d + de);
-            const float q2 = fmaxf(fmaf(ne * ne, c2, D), 1e-30f);
-            const float iq = rsqrt_approx(q2), q = q2 * iq;
-            aR = fmaf(wt, -D * iq * rcp_approx(fmaf(ne, c0, q)), aR);
-            aT = fmaf(wt, (c2 * (fmaf(d, d, 2.0f * d) - de) * (n2 + ne) - D) * iq * rcp_approx(fmaf(n2, c0, q)), aT);
-            aX = fmaf(wt, v.z * iq, aX);
-            aA = fmaf(wt, v.w * iq, aA);
+        for (int g = 0; g < 16; g += 2) {
+            const float4 v = __ldg(p + g), w = __ldg(p + g + 1);
+            const float2 d = make_float2(v.z, v.w);
+            add(make_float2(v.x, v.y), d, __fadd2_rn(two(1.0f), d), make_float2(w.x, w.y), make_float2(w.z, w.w));
         }
         x0 = xb;
     }
@@ -189,24 +205,23 @@ static __device__ __noinline__ float4 exact_fields_planar(const AtmParams* __res
         // unrolled: the points' special-function chains overlap (a few photons beyond the
         // tables leave one warp to integrate them, so latency, not issue, sets its time)
 #pragma unroll
-        for (int g = 0; g < 16; ++g) {
-            const float gx = c_gl16_x[g & 7], y = (g < 8) ? fmaf(-half, gx, mid) : fmaf(half, gx, mid);
-            const float wt = half * c_gl16_w[g & 7];
-            const float d = piece_delta<decltype(lin)::value>(law, y);
+        for (int g = 0; g < 16; g += 2) {
+            const int i = g & 7;
+            const float2 y = __ffma2_rn(two(g < 8 ? -half : half), make_float2(c_gl16_x[i], c_gl16_x[i + 1]), two(mid));
+            const float2 wt = __fmul2_rn(two(half), make_float2(c_gl16_w[i], c_gl16_w[i + 1]));
+            const float2 d = make_float2(piece_delta<decltype(lin)::value>(law, y.x), piece_delta<decltype(lin)::value>(law, y.y));
+            float2 X = two(0.0f), A = two(0.0f);
+            if (trans) {
+                const float2 e = __fmul2_rn(two(ap.aer_c2), y);
+                X = __fmul2_rn(two(ap.rho_per_delta), d);
+                A = __fmul2_rn(two(ap.aer_hobs), make_float2(ex2_approx(e.x), ex2_approx(e.y)));
+            }
             if (refr) {
-                const float n = 1.0f + d, n2 = n * n;
-                const float D = (d - de) * (2.0f + d + de);
-                const float q2 = fmaxf(fmaf(ne * ne, c2, D), 1e-30f);
-                const float iq = rsqrt_approx(q2), q = q2 * iq;
-                aR = fmaf(wt, -D * iq * rcp_approx(fmaf(ne, c0, q)), aR);
-                aT = fmaf(wt, (c2 * (fmaf(d, d, 2.0f * d) - de) * (n2 + ne) - D) * iq * rcp_approx(fmaf(n2, c0, q)), aT);
-                if (trans) {
-                    aX = fmaf(wt, ap.rho_per_delta * d * n * iq, aX);
-                    aA = fmaf(wt, ap.aer_hobs * ex2_approx(ap.aer_c2 * y) * n * iq, aA);
-                }
+                const float2 n = __fadd2_rn(two(1.0f), d);
+                add(wt, d, n, __fmul2_rn(X, n), __fmul2_rn(A, n));
             } else if (trans) {
-                aX = fmaf(wt, ap.rho_per_delta * d, aX);
-                aA = fmaf(wt, ap.aer_hobs * ex2_approx(ap.aer_c2 * y), aA);
+                aX = fmaf(wt.y, X.y, fmaf(wt.x, X.x, aX));
+                aA = fmaf(wt.y, A.y, fmaf(wt.x, A.x, aA));
             }
         }
         xa = xb;

@@ -539,7 +539,6 @@ __device__ __noinline__ float4 snell_path(const AtmParams& ap, float dz, float c
         for_slabs(ns, slab);
     } else {
         // two slabs at a time in packed FP32 instructions, each in the operations and order of `slab`
-        auto two = [](float v) { return make_float2(v, v); };
         const bool layered = ap.kind == CS_ATM_LAYERED;
         const float nsf = (float)ns;
         float2 j = make_float2(0.5f, 1.5f);   // index + 1/2
