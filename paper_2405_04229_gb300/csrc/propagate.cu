@@ -717,7 +717,7 @@ __device__ __forceinline__ float transmission_T(const AtmParams& ap, float GX, f
 // The correction fields at (dz, tan^2 of the local zenith) and the
 // transmission: the network's outputs where it applies, else the bilinear
 // table lookup; (0, 0, 1) without tables.
-template <bool SURR, int FIX>
+template <int SURR, int FIX>
 __device__ __forceinline__ void correction_fields(const AtmParams& ap, bool use_net, const float (&net)[3], float dz,
                                                   float w, float inv_l, float inv_uz, float& GR, float& Gt,
                                                   float& Tr) {
@@ -753,10 +753,13 @@ __device__ __forceinline__ void correction_fields(const AtmParams& ap, bool use_
     if (!(FIX || ap.transmission)) Tr = 1.0f;
 }
 
+// SURR: the tables, the network with single activations, or with split ones (its instances of their
+// own: both forms in one spilled, and the split one wants its block's 128 registers a thread).
+enum { kNoNet = 0, kNet = 1, kNetSplit = 2 };
 // The network as a kernel parameter, nothing in the other instances.
 struct NoNet {};
-template <bool SURR>
-using NetParam = std::conditional_t<SURR, SurrogateNet, NoNet>;
+template <int SURR>
+using NetParam = std::conditional_t<SURR != kNoNet, SurrogateNet, NoNet>;
 
 // Stages 3-5 for one bunch: generation on the cone (Sec. 4.2), the upward
 // filter (Sec. 5.3.4), straight line (Eq. 3.3; on the sphere, the vacuum
@@ -775,10 +778,10 @@ enum { kModeMain = 0, kModeCheck = 1, kModeExact = 2 };
 // FIX: the launch configuration as compile-time constants instead of parameter tests, whose uniform
 // branches cost issue slots.  kFixed, kFixedOptics: refraction, transmission and tables on,
 // histogram, telescopes and time sums on, without and with camera optics (the LV3 switch stays a
-// test; the network with single activations); kAny: tested.  1e6 segments: optics 252 -> 233 us,
-// fluorescence 177 -> 168 us, the network 946 -> 847 us (its two forms in one instance spilled).
+// test; of the network, the single form only); kAny: tested.  1e6 segments: optics 252 -> 233 us,
+// fluorescence 177 -> 168 us, the network 946 -> 847 us.
 enum { kAny = 0, kFixed = 1, kFixedOptics = 2 };
-template <bool SURR, bool SPH, bool REC, bool FL, bool TR, int MODE = kModeMain, int FIX = kAny, typename SM>
+template <int SURR, bool SPH, bool REC, bool FL, bool TR, int MODE = kModeMain, int FIX = kAny, typename SM>
 __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, long long base,
                                       const PropParams& pp, const AtmParams& ap, const DetParams& dp,
                                       const OutParams& op, const NetParam<SURR>& sv, TcSmem<kThreadsSur / 128>* tcs,
@@ -869,7 +872,7 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                             use_net ? fmaf(sv.in_scale[1], cos_z, sv.in_shift[1]) : 0.0f,
                             use_net ? fmaf(sv.in_scale[2], inv_l, sv.in_shift[2]) : 0.0f};
         float y[3];
-        const bool ok = !FIX && sv.split ? net128_tc<true>(sv, *tcs, x, y) : net128_tc<false>(sv, *tcs, x, y);
+        const bool ok = net128_tc<SURR == kNetSplit>(sv, *tcs, x, y);
         use_net = use_net && ok;   // a tensor-core wait that gave up: the tables take over
         if (use_net) {   // the network's part plus the first-order baseline
             const float3 bl = surrogate_baseline(sv, dz, cos_z, inv_l);
@@ -1341,7 +1344,7 @@ __device__ __forceinline__ void mark_group(unsigned int* scratch, long long n_wt
 // whose bit the photon kernel left clear, regenerates the sub-steps and
 // bunches of the others from their keyed draws, and propagates the bunches
 // beyond the tables along the exact path, 32 at a time per warp.
-template <bool SURR, bool SPH, int MINB, bool REC, bool FL = false, bool TR = false, bool EX = false,
+template <int SURR, bool SPH, int MINB, bool REC, bool FL = false, bool TR = false, bool EX = false,
           int FIX = kAny, int NT = SURR ? kThreadsSur : kThreads>
 __global__ void __launch_bounds__(NT, MINB)
 propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, const OutParams op,
@@ -1498,7 +1501,7 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                     const int ib = p0 + lane - W.first[j];
                     if constexpr (!EX) {
                         if (in && (!TR || ((p0 >> 5) & (parts - 1)) == part)) {
-                            const bool bey = bunch<false, SPH, REC, FL, TR, kModeMain, FIX>(W, j, ib, true, base, pp, ap,
+                            const bool bey = bunch<kNoNet, SPH, REC, FL, TR, kModeMain, FIX>(W, j, ib, true, base, pp, ap,
                                                                                            dp, op, sv, tcs, T);
                             // a bunch beyond the tables goes to the exact pass's queue (one
                             // reservation per group of converged lanes); when the queue is full its
@@ -1528,7 +1531,7 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                         // bunches beyond the tables are queued and propagated 32 at a time, so that
                         // the warp stays converged
                         const bool last = p0 + 32 >= M;
-                        const bool take = in && bunch<false, SPH, REC, FL, TR, kModeCheck>(W, j, ib, true, base, pp, ap, dp,
+                        const bool take = in && bunch<kNoNet, SPH, REC, FL, TR, kModeCheck>(W, j, ib, true, base, pp, ap, dp,
                                                                                           op, sv, tcs, T);
                         const unsigned int m = __ballot_sync(0xffffffffu, take);
                         if (take) {
@@ -1541,7 +1544,7 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                             const int n_run = min(nq, 32);
                             if (lane < n_run) {
                                 const int e = nq - n_run + lane;
-                                bunch<false, SPH, REC, FL, TR, kModeExact>(W, W.q_sub[e], W.q_bunch[e], true, base, pp, ap, dp,
+                                bunch<kNoNet, SPH, REC, FL, TR, kModeExact>(W, W.q_sub[e], W.q_bunch[e], true, base, pp, ap, dp,
                                                                            op, sv, tcs, T);
                             }
                             nq -= n_run;
@@ -1630,7 +1633,7 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                     const long long base_l = li - lane;   // so that base + slot is the segment's index
                     import_segment<SPH, FL>(W, lane, pp.segs + li, pp, ap, dp, invalid, dropped, false);
                     substep<SPH, FL>(W, W.sub[lane], lane, (int)ent.z, base_l, pp, ap);
-                    bunch<false, SPH, REC, FL, TR, kModeExact>(W, lane, (int)ent.w, true, base_l, pp, ap, dp, op, sv, tcs, T);
+                    bunch<kNoNet, SPH, REC, FL, TR, kModeExact>(W, lane, (int)ent.w, true, base_l, pp, ap, dp, op, sv, tcs, T);
                 }
             }
             __syncwarp();
@@ -1856,13 +1859,13 @@ cs_status launch_kernel(unsigned grid, cudaStream_t stream, const PropParams& pp
         constexpr bool S = decltype(sph)::value, F = decltype(fl)::value, T = decltype(tr)::value;
         if constexpr (!T) {
             if (fix && !rec)
-                return cam ? go(propagate_kernel<false, S, 4, false, F, false, false, kFixedOptics>, kThreads)
-                           : go(propagate_kernel<false, S, 4, false, F, false, false, kFixed>, kThreads);
+                return cam ? go(propagate_kernel<kNoNet, S, 4, false, F, false, false, kFixedOptics>, kThreads)
+                           : go(propagate_kernel<kNoNet, S, 4, false, F, false, false, kFixed>, kThreads);
         }
         if constexpr (!F && !T) {
-            if (fix && !cam) return go(propagate_kernel<false, S, 4, true, false, false, false, kFixed>, kThreads);
+            if (fix && !cam) return go(propagate_kernel<kNoNet, S, 4, true, false, false, false, kFixed>, kThreads);
         }
-        rec ? go(propagate_kernel<false, S, 4, true, F, T>, kThreads) : go(propagate_kernel<false, S, 4, false, F, T>, kThreads);
+        rec ? go(propagate_kernel<kNoNet, S, 4, true, F, T>, kThreads) : go(propagate_kernel<kNoNet, S, 4, false, F, T>, kThreads);
     };
     using t_ = std::true_type;
     using f_ = std::false_type;
@@ -1870,8 +1873,9 @@ cs_status launch_kernel(unsigned grid, cudaStream_t stream, const PropParams& pp
     if (sur) {
         auto network = [&](auto sph) {
             constexpr bool S = decltype(sph)::value;
-            if (fix && !cam && !rec && !net.split) go_net(propagate_kernel<true, S, 2, false, false, false, false, kFixed>);
-            else rec ? go_net(propagate_kernel<true, S, 2, true>) : go_net(propagate_kernel<true, S, 2, false>);
+            if (net.split) rec ? go_net(propagate_kernel<kNetSplit, S, 1, true>) : go_net(propagate_kernel<kNetSplit, S, 1, false>);
+            else if (fix && !cam && !rec) go_net(propagate_kernel<kNet, S, 2, false, false, false, false, kFixed>);
+            else rec ? go_net(propagate_kernel<kNet, S, 2, true>) : go_net(propagate_kernel<kNet, S, 2, false>);
         };
         ap.spherical ? network(t_{}) : network(f_{});
     } else if (ap.spherical) {
@@ -1889,11 +1893,11 @@ cs_status launch_kernel(unsigned grid, cudaStream_t stream, const PropParams& pp
         const unsigned grid_x = (unsigned)std::max<long long>(1, std::min<long long>(n_wtiles, (long long)device_sm_count() * 4));
         auto pass = [&](auto kernel) { dependent(kernel, grid_x, kThreads, kSmemPass, NoNet{}); };
         if (ap.spherical) {
-            if (fl) rec ? pass(propagate_kernel<false, true, 4, true, true, false, true>) : pass(propagate_kernel<false, true, 4, false, true, false, true>);
-            else rec ? pass(propagate_kernel<false, true, 4, true, false, false, true>) : pass(propagate_kernel<false, true, 4, false, false, false, true>);
+            if (fl) rec ? pass(propagate_kernel<kNoNet, true, 4, true, true, false, true>) : pass(propagate_kernel<kNoNet, true, 4, false, true, false, true>);
+            else rec ? pass(propagate_kernel<kNoNet, true, 4, true, false, false, true>) : pass(propagate_kernel<kNoNet, true, 4, false, false, false, true>);
         } else {
-            if (fl) rec ? pass(propagate_kernel<false, false, 4, true, true, false, true>) : pass(propagate_kernel<false, false, 4, false, true, false, true>);
-            else rec ? pass(propagate_kernel<false, false, 4, true, false, false, true>) : pass(propagate_kernel<false, false, 4, false, false, false, true>);
+            if (fl) rec ? pass(propagate_kernel<kNoNet, false, 4, true, true, false, true>) : pass(propagate_kernel<kNoNet, false, 4, false, true, false, true>);
+            else rec ? pass(propagate_kernel<kNoNet, false, 4, true, false, false, true>) : pass(propagate_kernel<kNoNet, false, 4, false, false, false, true>);
         }
         CS_CUDA_TRY(cudaGetLastError());
     }
@@ -1903,17 +1907,29 @@ cs_status launch_kernel(unsigned grid, cudaStream_t stream, const PropParams& pp
 template <bool S, bool F, bool T>
 cudaError_t set_exact_smem(int smem) {
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    cudaError_t e = cudaFuncSetAttribute(propagate_kernel<false, S, 4, false, F, T>, attr, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<false, S, 4, true, F, T>, attr, smem);
+    cudaError_t e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, false, F, T>, attr, smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, true, F, T>, attr, smem);
     if (!T) {   // the exact pass of the table-tracer instances
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<false, S, 4, false, F, false, true>, attr, (int)kSmemPass);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<false, S, 4, true, F, false, true>, attr, (int)kSmemPass);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, false, F, false, true>, attr, (int)kSmemPass);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, true, F, false, true>, attr, (int)kSmemPass);
     }
     if (!T) {   // the fixed-configuration instances
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<false, S, 4, false, F, false, false, kFixed>, attr, smem);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<false, S, 4, false, F, false, false, kFixedOptics>, attr, smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, false, F, false, false, kFixed>, attr, smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, false, F, false, false, kFixedOptics>, attr, smem);
     }
-    if (!T && !F && e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<false, S, 4, true, false, false, false, kFixed>, attr, smem);
+    if (!T && !F && e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, true, false, false, false, kFixed>, attr, smem);
+    return e;
+}
+
+template <bool S>
+cudaError_t set_network_smem() {
+    const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const int one = (int)smem_surrogate(false), split = (int)smem_surrogate(true);
+    cudaError_t e = cudaFuncSetAttribute(propagate_kernel<kNet, S, 2, false>, attr, one);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNet, S, 2, true>, attr, one);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNet, S, 2, false, false, false, false, kFixed>, attr, one);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNetSplit, S, 1, false>, attr, split);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNetSplit, S, 1, true>, attr, split);
     return e;
 }
 
@@ -1928,8 +1944,7 @@ cs_status set_smem_attributes() {
     if (dev < 0 || dev >= kMaxDevices) return CS_ERR_INVALID_ARG;
     std::lock_guard<std::mutex> lock(g_attr_mu);
     if (g_attr_done[dev]) return CS_OK;
-    const int smem = (int)kSmemExact, smem_sur = (int)smem_surrogate(true);
-    const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    const int smem = (int)kSmemExact;
     CS_CUDA_TRY((set_exact_smem<false, false, false>(smem)));
     CS_CUDA_TRY((set_exact_smem<false, false, true>(smem)));
     CS_CUDA_TRY((set_exact_smem<false, true, false>(smem)));
@@ -1938,12 +1953,8 @@ cs_status set_smem_attributes() {
     CS_CUDA_TRY((set_exact_smem<true, false, true>(smem)));
     CS_CUDA_TRY((set_exact_smem<true, true, false>(smem)));
     CS_CUDA_TRY((set_exact_smem<true, true, true>(smem)));
-    CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, false, 2, false>, attr, smem_sur));
-    CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, false, 2, false, false, false, false, kFixed>, attr, smem_sur));
-    CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, true, 2, false, false, false, false, kFixed>, attr, smem_sur));
-    CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, false, 2, true>, attr, smem_sur));
-    CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, true, 2, false>, attr, smem_sur));
-    CS_CUDA_TRY(cudaFuncSetAttribute(propagate_kernel<true, true, 2, true>, attr, smem_sur));
+    CS_CUDA_TRY(set_network_smem<false>());
+    CS_CUDA_TRY(set_network_smem<true>());
     g_attr_done[dev] = true;
     return CS_OK;
 }
