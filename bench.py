@@ -327,7 +327,7 @@ def run_batched(args):
                        "segments": n, "photons_per_step": photons, "bunch_sizes": per_shower_bunch,
                        "blocks_per_sm": tune.blocks_per_sm, "tiling_ms": [round(tune.ms[i], 3) for i in range(4)],
                        "generation_s": round(gen_s, 1), "l2": "inputs (%.1f GB) larger than L2" % (arr.nbytes / 1e9)},
-            "counters": [int(x) for x in h["counters"]], "cpu_baseline": cpu, "gpu_launches": 2 * args.steps,
+            "counters": [int(x) for x in h["counters"]], "cpu_baseline": cpu, "gpu_launches": 3 * args.steps,
             "clocks": clk.summary()}
     if getattr(args, "quiet", False):
         return line
@@ -584,7 +584,7 @@ def run_inclined(args):
                          "frac": achieved / peak, "traffic": kernel_profile("propagate_kernel_spherical_traffic.txt")[0],
                          "note": "per chunk launch; spherical lane-op count per bunch %d" % OPS_PER_BUNCH_SPHERICAL},
             "kernel_ms": k_ms, "cpu_baseline": cpu, "surrogate": surrogate, "e2e": e2e, "lv1_filter": lv1_res, "lv3_filter": lv3_res,
-            "gpu_launches": 2 * args.steps * n_chunks, "clocks": clk.summary()}
+            "gpu_launches": 3 * args.steps * n_chunks, "clocks": clk.summary()}
     if getattr(args, "quiet", False):
         return line
     print(json.dumps(line), flush=True)
@@ -1001,7 +1001,7 @@ def main():
             "snell_tracer": snell,
             "fluorescence": fluor,
             "e2e": e2e,
-            "gpu_launches": 2 * args.steps,   # the photon kernel and its exact pass, per step
+            "gpu_launches": 3 * args.steps,   # per step: the zeroing, the photon kernel and its exact pass
             "clocks": sm_clk,
         }
         if configs:
