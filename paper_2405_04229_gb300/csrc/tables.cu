@@ -161,6 +161,23 @@ __global__ void piece_points_kernel(AtmF64 a, const int* begin, PiecePoint* pt) 
     for (int i = threadIdx.x; i < piece.n; i += blockDim.x) pt[begin[p] + i] = piece.at(a, i);
 }
 
+// Calls add(point) for the points from h_obs up to the last of the nc cuts, in order.
+template <typename F>
+__device__ __forceinline__ void for_points(const AtmF64& a, const PieceTable& tab, const double* cuts, int nc, F&& add) {
+    int p = 0;
+    for (; p + 2 < nc && p < tab.n; ++p) {
+        const int end = __ldg(tab.begin + p + 1);
+        for (int i = __ldg(tab.begin + p); i < end; ++i) {
+            const PiecePoint* q = tab.pt + i;
+            add(PiecePoint{__ldg(&q->h), __ldg(&q->wt), __ldg(&q->d), __ldg(&q->rho), __ldg(&q->ea)});
+        }
+    }
+    for (; p + 1 < nc; ++p) {
+        const Piece piece(a, cuts[p], cuts[p + 1]);
+        for (int i = 0; i < piece.n; ++i) add(piece.at(a, i));
+    }
+}
+
 // The four integrals from h_obs up to h_e for zenith theta0 (cos0, sin0),
 // normalised as described in common.cuh.  The FP64 pipe bounds it (88 % busy):
 // the points of whole pieces come from the table, divisions by one number
@@ -208,18 +225,7 @@ __device__ void node_fields(const AtmF64& a, const PieceTable& tab, double h_e, 
             }
         }
     };
-    int p = 0;
-    for (; p + 2 < nc && p < tab.n; ++p) {
-        const int end = __ldg(tab.begin + p + 1);
-        for (int i = __ldg(tab.begin + p); i < end; ++i) {
-            const PiecePoint* q = tab.pt + i;
-            add(PiecePoint{__ldg(&q->h), __ldg(&q->wt), __ldg(&q->d), __ldg(&q->rho), __ldg(&q->ea)});
-        }
-    }
-    for (; p + 1 < nc; ++p) {
-        const Piece piece(a, cuts[p], cuts[p + 1]);
-        for (int i = 0; i < piece.n; ++i) add(piece.at(a, i));
-    }
+    for_points(a, tab, cuts, nc, add);
     if (a.spherical) {
         // G_R = (arc length correction on the ground sphere) cos^3 / sin, G_t = c dt cos,
         // G_X = X cos, G_A = A cos
@@ -288,43 +294,20 @@ __global__ void assemble_kernel(const double* F, const double* Fb, const int* be
 // Vertical integrals from h_obs up to each height h (one thread per height):
 // {int (n - 1) dh [m], n(h) - 1 (from above), int 100 rho dh [g/cm^2],
 //  int exp(-h / H_A) dh [m]}, by the same Gauss-Legendre pieces as the tables.
-__global__ void column_kernel(AtmF64 a, const double* h_in, size_t n, Fields4* out) {
+__global__ void column_kernel(AtmF64 a, PieceTable tab, const double* h_in, size_t n, Fields4* out) {
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double h = h_in[i];
     double de, rho_e;
     delta_rho(a, h, false, &de, &rho_e);
     double cuts[kMaxNodes + 3];
-    int nc = 0;
-    cuts[nc++] = a.h_obs;
-    if (a.kind == CS_ATM_LAYERED) {
-        for (int k = 1; k < a.n_layers; ++k)
-            if (a.lay_h[k] > a.h_obs && a.lay_h[k] < h) cuts[nc++] = a.lay_h[k];
-        if (a.h_top > a.h_obs && a.h_top < h) cuts[nc++] = a.h_top;
-    } else if (a.kind == CS_ATM_LINEAR) {
-        if (a.lin_h1 > a.h_obs && a.lin_h1 < h) cuts[nc++] = a.lin_h1;
-    } else if (a.kind == CS_ATM_TABLE) {
-        for (int k = 1; k < a.n_nodes; ++k)
-            if (a.node_h[k] > a.h_obs && a.node_h[k] < h) cuts[nc++] = a.node_h[k];
-    }
-    cuts[nc++] = h;
+    const int nc = piece_cuts(a, h, cuts);
     double sI = 0.0, sX = 0.0, sA = 0.0;
-    for (int piece = 0; piece + 1 < nc; ++piece) {
-        const double lo = cuts[piece], hi = cuts[piece + 1];
-        const int nsub = (int)ceil((hi - lo) / kSubMax);
-        const double step = (hi - lo) / nsub;
-        for (int sub = 0; sub < nsub; ++sub) {
-            const double mid = lo + (sub + 0.5) * step, half = 0.5 * step;
-            for (int g = 0; g < kGL; ++g) {
-                const double y = mid + half * c_gl_x[g], wt = half * c_gl_w[g];
-                double d, rho;
-                delta_rho(a, y, false, &d, &rho);
-                sI += wt * d;
-                sX += wt * 100.0 * rho;
-                sA += wt * exp(-y / a.H_A);
-            }
-        }
-    }
+    for_points(a, tab, cuts, nc, [&](const PiecePoint& v) {
+        sI += v.wt * v.d;
+        sX += v.wt * 100.0 * v.rho;
+        sA += v.wt * v.ea;
+    });
     out[i] = Fields4{sI, de, sX, sA};
 }
 
@@ -675,7 +658,9 @@ extern "C" cs_status cs_atmosphere_create(const cs_atmosphere_desc* d, cs_atmosp
 namespace cs {
 cs_status column_fields(const cs_atmosphere* atm, const double* d_h, size_t n, Fields4* d_out, cudaStream_t stream) {
     if (n == 0) return CS_OK;
-    column_kernel<<<(unsigned)((n + 127) / 128), 128, 0, stream>>>(atm->f64, d_h, n, d_out);
+    // one warp a block: the heights are few (4,096), the FP64 pipe of each SM narrow (with the points of
+    // whole pieces from the table, a training 20.3 -> 19.95 ms)
+    column_kernel<<<(unsigned)((n + 31) / 32), 32, 0, stream>>>(atm->f64, piece_table(atm), d_h, n, d_out);
     CS_CUDA_TRY(cudaGetLastError());
     return CS_OK;
 }
