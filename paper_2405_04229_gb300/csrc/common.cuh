@@ -168,6 +168,7 @@ struct PropParams {
     uint32_t rk[20];   // Philox key schedule: round r uses rk[2r], rk[2r + 1]
     int tile_segs;     // segments a warp takes at a time (at most 32; the exact tracer)
     int parts_log2;    // the stepper: log2 of the parts that a tile's bunch rounds are dealt out in
+    int one_round;     // the exact tracer: every resident warp has at most one tile (or part); see ONE
     int tiles_per_bit; // warp tiles (32 segments) per bit of the exact pass's tile map
     unsigned int q_cap; // entries of the exact pass's bunch queue (0: tile map only)
     unsigned int q_off; // its offset in the scratch, in 32-bit words (a multiple of 4)

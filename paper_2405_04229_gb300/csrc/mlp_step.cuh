@@ -6,9 +6,10 @@
 // products and its partial sums; reduce_kernel adds them in a fixed order and
 // applies Adam.  As 27 launches through global memory (GEMMs that re-stage
 // their operands, elementwise passes between them) a step of 32,768 rows took
-// 260 us; in this form 35 + 14 us.  What bounds it: latency -- 16 warps per SM
-// (35 % of issue slots) evaluate 192 tanh a row twice and store the operands
-// between seven MMA round trips and their barriers.
+// 260 us; in this form 31 + 11 us.  What bounds it: latency -- 16 warps per SM
+// (23 % of issue slots) evaluate 192 tanh a row twice and store the operands
+// between seven MMA round trips and their barriers.  (1,024 threads, four per
+// row, took the same time.)
 //
 // Arithmetic and its order are the unfused path's: the same BF16 hi + lo
 // splits, the same K = 16 products in the same order, partial sums over the

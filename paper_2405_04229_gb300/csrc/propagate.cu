@@ -1343,9 +1343,9 @@ __device__ __forceinline__ void mark_group(unsigned int* scratch, long long n_wt
 // instances only): the exact pass walks the same warp tiles, skips those
 // whose bit the photon kernel left clear, regenerates the sub-steps and
 // bunches of the others from their keyed draws, and propagates the bunches
-// beyond the tables along the exact path, 32 at a time per warp.
+// beyond the tables along the exact path, 32 at a time per warp.  ONE: see below.
 template <int SURR, bool SPH, int MINB, bool REC, bool FL = false, bool TR = false, bool EX = false,
-          int FIX = kAny, int NT = SURR ? kThreadsSur : kThreads>
+          int FIX = kAny, bool ONE = false, int NT = SURR ? kThreadsSur : kThreads>
 __global__ void __launch_bounds__(NT, MINB)
 propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, const OutParams op,
                  unsigned int* scratch, const NetParam<SURR> sv) {
@@ -1355,7 +1355,12 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
     // photon kernel's retire.  Both wait here for the completion (and the memory) of the kernel
     // before; the photon kernel lets the exact pass launch from the start.  Without the launch
     // attribute these instructions are no-ops.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    // A launch of one round (ONE: every warp has at most one tile) takes no tile from the scratch and
+    // waits only before its first bunch, so that import and sub-steps overlap the zeroing (the segments
+    // are complete: the zeroing kernel itself starts after everything before it).  1,000 straight
+    // tracks 15.4 -> 13.8 us a call, 5,003 segments of bunch 1 29.2 -> 27.0 us; as a test at run time in
+    // the instances of larger launches it cost those 1 %.
+    if (!ONE) asm volatile("griddepcontrol.wait;" ::: "memory");
     if (!EX) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (EX && __ldcg(scratch + 2) == 0 && __ldcg(scratch + 3) == 0) return;   // no bunch beyond the tables
     unsigned int* const tile_ctr = scratch + (EX ? 1 : 0);
@@ -1492,6 +1497,7 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
                 // bunch, written by loops over the sub-steps, took 588 warp instructions per tile of
                 // 310 bunches, these look-ups about 130.)
                 int j_cur = -1, nq = 0;
+                if (ONE) asm volatile("griddepcontrol.wait;" ::: "memory");
                 for (int p0 = 0; p0 < M; p0 += 32) {
                     const unsigned int rel = (unsigned int)(W.first[j_cur + 1 + lane] - p0);
                     const unsigned int starts = __reduce_or_sync(0xffffffffu, rel < 32u ? 1u << rel : 0u);
@@ -1564,19 +1570,24 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
             // warp's place in the grid, without the counter, cost two registers and 1-2 % of C2.)
             for (;;) {
                 unsigned int wt = 0;
-                if (lane == 0) wt = atomicAdd(tile_ctr, 1u);
-                wt = __shfl_sync(0xffffffffu, wt, 0);
+                if (ONE) {   // a tile (part) per warp: no trips to the counter
+                    wt = blockIdx.x * (unsigned int)(NT / 32) + (unsigned int)(t >> 5);
+                } else {
+                    if (lane == 0) wt = atomicAdd(tile_ctr, 1u);
+                    wt = __shfl_sync(0xffffffffu, wt, 0);
+                }
                 const long long base = (long long)(TR ? wt >> pp.parts_log2 : wt) * pp.tile_segs;
                 if (base >= pp.n) break;
                 const int part = TR ? (int)(wt & ((1u << pp.parts_log2) - 1u)) : 0;
                 // some warp takes the tile one round of the grid ahead about a tile's time from now:
                 // its segments into L2 (the counter is not advanced: a reserved tile would wait for
                 // a slow warp at the end of the launch)
-                if (!TR) {
+                if (!TR && !ONE) {
                     const long long ahead = base + (long long)(gridDim.x * (kThreads / 32)) * pp.tile_segs + lane;
                     if (ahead < pp.n) asm volatile("prefetch.global.L2 [%0];" ::"l"(pp.segs + ahead));
                 }
                 process_tile(base, (int)std::min<long long>(pp.tile_segs, pp.n - base), part, 1 << pp.parts_log2);
+                if (ONE) break;
             }
         } else {
             // the exact pass takes the queued bunches a block's worth at a time, then the marked groups
@@ -1728,6 +1739,7 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
     }
 
     if (SURR) tc_teardown(*tcs);
+    if (ONE) asm volatile("griddepcontrol.wait;" ::: "memory");   // (a warp without a bunch)
     if (EX) {   // the photon kernel counted these segments and their emitted bunches
         emitted = 0;
         invalid = 0;
@@ -1857,6 +1869,11 @@ cs_status launch_kernel(unsigned grid, cudaStream_t stream, const PropParams& pp
     const bool cam = dp.cam_n > 0;
     auto exact = [&](auto sph, auto fl, auto tr) {
         constexpr bool S = decltype(sph)::value, F = decltype(fl)::value, T = decltype(tr)::value;
+        if constexpr (!F && !T) {
+            if (pp.one_round && !rec && !cam)
+                return fix ? go(propagate_kernel<kNoNet, S, 4, false, false, false, false, kFixed, true>, kThreads)
+                           : go(propagate_kernel<kNoNet, S, 4, false, false, false, false, kAny, true>, kThreads);
+        }
         if constexpr (!T) {
             if (fix && !rec)
                 return cam ? go(propagate_kernel<kNoNet, S, 4, false, F, false, false, kFixedOptics>, kThreads)
@@ -1917,7 +1934,11 @@ cudaError_t set_exact_smem(int smem) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, false, F, false, false, kFixed>, attr, smem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, false, F, false, false, kFixedOptics>, attr, smem);
     }
-    if (!T && !F && e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, true, false, false, false, kFixed>, attr, smem);
+    if (!T && !F) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, true, false, false, false, kFixed>, attr, smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, false, false, false, false, kFixed, true>, attr, smem);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, false, false, false, false, kAny, true>, attr, smem);
+    }
     return e;
 }
 
@@ -1978,11 +1999,12 @@ int default_blocks_per_sm(const cs_opts& o) {
 // Parts (the stepper only: a round of bunches then takes ~20 times the tile's own work, so that
 // repeating import and sub-steps in up to 16 warps costs little): enough for eight units per
 // resident warp.  1,000 / 10,000 / 100,000 segments of bunch 5: 0.77 / 0.94 / 3.74 ms against
-// 4.69 / 4.90 / 5.67 ms with whole tiles.
+// 4.69 / 4.90 / 5.67 ms with whole tiles (with the slab loop of that time; 100,000 take 0.74 ms now).
 unsigned int plan_launch(PropParams& pp, size_t n, const cs_opts& o) {
     const long long blocks = (long long)device_sm_count() * default_blocks_per_sm(o);
     pp.tile_segs = kWTile;
     pp.parts_log2 = 0;
+    pp.one_round = 0;
     if (o.surrogate) return (unsigned int)std::max<long long>(1, std::min<long long>(((long long)n + kTile - 1) / kTile, blocks));
     constexpr int wpb = kThreads / 32;   // warps per block
     const long long slots = blocks * wpb;
@@ -1995,6 +2017,7 @@ unsigned int plan_launch(PropParams& pp, size_t n, const cs_opts& o) {
         while (pp.tile_segs > 1 && pp.tile_segs > best * 1.5) pp.tile_segs >>= 1;
     }
     const long long units = (((long long)n + pp.tile_segs - 1) / pp.tile_segs) << pp.parts_log2;
+    pp.one_round = units <= slots;
     return (unsigned int)std::max<long long>(1, std::min<long long>((units + wpb - 1) / wpb, blocks));
 }
 
