@@ -366,8 +366,10 @@ __device__ __forceinline__ void hist_add(const OutParams& op, unsigned int key, 
 // zenith range (`hashed`) test the entries of their grid cell in the list for
 // their own sine squared s2: cell_delta(entry, corner_x, corner_y, ddx, ddy,
 // ddz) gives the centre minus the ground point.  Steeper arrivals test every
-// sphere through full_delta(index, ddx, ddy, ddz, radius).
-template <typename CellDelta, typename FullDelta>
+// sphere through full_delta(index, ddx, ddy, ddz, radius), AHEAD spheres' loads
+// at a time: eight in the exact pass, where a few such arrivals leave a few
+// warps to wait for each load (the inclined chunk 1335 -> 1313 us a call).
+template <int AHEAD, typename CellDelta, typename FullDelta>
 __device__ __forceinline__ int hit_telescope(const DetParams& dp, const TelHash& H, bool hashed, float s2, float x, float y,
                                              float ugx, float ugy, float ugz, CellDelta cell_delta, FullDelta full_delta) {
     int best = -1;
@@ -396,6 +398,7 @@ __device__ __forceinline__ int hit_telescope(const DetParams& dp, const TelHash&
         }
         return best >= 0 ? __ldg(H.cell_tel + best) : -1;
     }
+#pragma unroll AHEAD
     for (int it = 0; it < dp.n_tel; ++it) {
         float ddx, ddy, ddz, r;
         full_delta(it, ddx, ddy, ddz, r);
@@ -983,7 +986,7 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                         const float c2 = fmaxf(1.0f - s2, 1e-30f);
                         ugz = -c2 * rsqrt_approx(c2);
                     }
-                    tel = hit_telescope(
+                    tel = hit_telescope<MODE == kModeExact ? 8 : 1>(
                         dp, H, hashed, s2, x, y, ux * sc, uy * sc, ugz,
                         [&](const float4& D, float cx0, float cy0, float& ddx, float& ddy, float& ddz) {
                             ddx = D.x - ((Cg.x - cx0) + (Cg.y + rx));
@@ -1087,7 +1090,7 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                 const bool lvl0 = sg2 <= dp.hash[0].sin2_max;
                 auto detect = [&](const TelHash& H, const bool hashed) {
                 {
-                    tel = hit_telescope(
+                    tel = hit_telescope<MODE == kModeExact ? 8 : 1>(
                         dp, H, hashed, sg2, xs, ys, ugx, ugy, ugz,
                         [&](const float4& D, float cx0, float cy0, float& ddx, float& ddy, float& ddz) {
                             ddx = D.x - ((x - cx0) + xl);
@@ -1268,7 +1271,7 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                             ddy = (T3.y - Gy) - Gyl;
                             ddz = (T3.z - Gz) - Gzl;
                         };
-                        tel = hit_telescope(
+                        tel = hit_telescope<MODE == kModeExact ? 8 : 1>(
                             dp, H, hashed, sg2, xs, ys, ugx, ugy, ugz,
                             [&](const float4& D, float, float, float& ddx, float& ddy, float& ddz) { delta3(D, ddx, ddy, ddz); },
                             [&](int it, float& ddx, float& ddy, float& ddz, float& r) {
