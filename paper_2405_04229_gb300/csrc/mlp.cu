@@ -586,7 +586,7 @@ eval_kernel(const __grid_constant__ SurrogateNet sv, const float4* __restrict__ 
     TcSmem<kEvalThreads / 128>& T = *reinterpret_cast<TcSmem<kEvalThreads / 128>*>(smem_raw);
     tc_setup(T, sv);
     // every thread of the block takes the same number of rounds
-    for (size_t base = (size_t)blockIdx.x * kEvalThreads; base < n; base += (size_t)gridDim.x * kEvalThreads) {
+    for (size_t base = (size_t)blockIdx.x * blockDim.x; base < n; base += (size_t)gridDim.x * blockDim.x) {
         const size_t i = base + threadIdx.x;
         const float4 v = i < n ? in[i] : make_float4(0.f, 1.f, 3.0e-3f, 0.f);   // dz, cos(theta0), 1/lambda_nm
         const float x[3] = {sv.in_scale[0] * height_coordinate(sv, v.x) + sv.in_shift[0],
@@ -616,10 +616,13 @@ cs_status run_eval(const SurrogateNet& sv, const float4* d_in, size_t n, float4*
     const int smem = (int)TcSmem<kEvalThreads / 128>::bytes(split);
     CS_CUDA_TRY(cudaFuncSetAttribute(split ? eval_kernel<true> : eval_kernel<false>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    const unsigned grid = (unsigned)std::min<size_t>((n + kEvalThreads - 1) / kEvalThreads,
-                                                     (size_t)device_sm_count() * (split ? 1 : 2));
-    if (split) eval_kernel<true><<<grid, kEvalThreads, smem, s>>>(sv, d_in, n, d_out, network_only);
-    else eval_kernel<false><<<grid, kEvalThreads, smem, s>>>(sv, d_in, n, d_out, network_only);
+    // few points: smaller blocks on more SMs (a block's round lasts longer the more warps share its SM)
+    const size_t slots = (size_t)device_sm_count() * (split ? 1 : 2);
+    unsigned threads = kEvalThreads;
+    while (threads > 128 && n <= slots * (threads / 2)) threads /= 2;
+    const unsigned grid = (unsigned)std::min<size_t>((n + threads - 1) / threads, slots);
+    if (split) eval_kernel<true><<<grid, threads, smem, s>>>(sv, d_in, n, d_out, network_only);
+    else eval_kernel<false><<<grid, threads, smem, s>>>(sv, d_in, n, d_out, network_only);
     CS_CUDA_TRY(cudaGetLastError());
     const bool timed_out = tc_take_timeout(s);
     CS_CUDA_TRY(cudaStreamSynchronize(s));
