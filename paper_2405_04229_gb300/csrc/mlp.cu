@@ -624,8 +624,8 @@ cs_status run_eval(const SurrogateNet& sv, const float4* d_in, size_t n, float4*
     if (split) eval_kernel<true><<<grid, threads, smem, s>>>(sv, d_in, n, d_out, network_only);
     else eval_kernel<false><<<grid, threads, smem, s>>>(sv, d_in, n, d_out, network_only);
     CS_CUDA_TRY(cudaGetLastError());
-    const bool timed_out = tc_take_timeout(s);
-    CS_CUDA_TRY(cudaStreamSynchronize(s));
+    bool timed_out = false;
+    CS_CUDA_TRY(tc_read_timeout(timed_out, s));
     return timed_out ? CS_ERR_TIMEOUT : CS_OK;
 }
 

@@ -41,16 +41,22 @@ struct TcSmem {
 // and cleared by that unit's host calls through tc_take_timeout().
 static __device__ unsigned int g_tc_timeout = 0;
 
-static inline bool tc_take_timeout(cudaStream_t s = nullptr) {   // (waits for the stream's work)
+// (Waits for the stream's work.)
+static inline cudaError_t tc_read_timeout(bool& timed_out, cudaStream_t s) {
     unsigned int v = 0;
-    if (cudaMemcpyFromSymbolAsync(&v, g_tc_timeout, sizeof v, 0, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-        return false;
-    if (v) {
+    cudaError_t e = cudaMemcpyFromSymbolAsync(&v, g_tc_timeout, sizeof v, 0, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess && v) {
         const unsigned int z = 0;
         cudaMemcpyToSymbol(g_tc_timeout, &z, sizeof z);
     }
-    return v != 0;
+    timed_out = e == cudaSuccess && v != 0;
+    return e;
+}
+
+static inline bool tc_take_timeout() {
+    bool timed_out = false;
+    return tc_read_timeout(timed_out, nullptr) == cudaSuccess && timed_out;
 }
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
