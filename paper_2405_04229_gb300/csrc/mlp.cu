@@ -616,7 +616,8 @@ cs_status run_eval(const SurrogateNet& sv, const float4* d_in, size_t n, float4*
     const int smem = (int)TcSmem<kEvalThreads / 128>::bytes(split);
     CS_CUDA_TRY(cudaFuncSetAttribute(split ? eval_kernel<true> : eval_kernel<false>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    // few points: smaller blocks on more SMs (a block's round lasts longer the more warps share its SM)
+    // few points: smaller blocks on more SMs (a block's round lasts longer the more warps share its SM;
+    // 60,000 points 38.5 -> 33 us a call against blocks of 256, 1,000 points 33 us with either)
     const size_t slots = (size_t)device_sm_count() * (split ? 1 : 2);
     unsigned threads = kEvalThreads;
     while (threads > 128 && n <= slots * (threads / 2)) threads /= 2;
