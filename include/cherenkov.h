@@ -526,7 +526,8 @@ cs_status cs_surrogate_info(const cs_surrogate* s, float* params, size_t n_param
 /* One forward and backward pass of the training path on B rows (host
  * arrays: params in the layout above, x and t B x 3 normalised): the loss
  * (1/B) sum (y - t)^2 and its gradient (host, same layout).  For checking
- * the tensor-core training kernels against a reference. */
+ * the tensor-core training kernels against a reference.  CS_ERR_TIMEOUT, and
+ * no gradients, if a wait on the tensor cores ran out. */
 cs_status cs_mlp_loss_grad(const float* params, const float* x, const float* t, int B, float* grad, float* loss);
 
 /* Allocation-free form of the device-pointer call (the thesis has no

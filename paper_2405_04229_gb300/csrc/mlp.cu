@@ -1117,12 +1117,17 @@ extern "C" cs_status cs_mlp_loss_grad(const float* params, const float* x, const
         cleanup();
         return CS_ERR_CUDA;
     }
-    cudaMemcpy(X, x, (size_t)B * 12, cudaMemcpyHostToDevice);
-    cudaMemcpy(T, t, (size_t)B * 12, cudaMemcpyHostToDevice);
-    cudaMemcpy(p, params, kNParams * 4, cudaMemcpyHostToDevice);
-    cudaMemset(g, 0, kNParams * 4);
-    cudaMemset(w.loss, 0, 4);
-    cudaError_t e = cudaSuccess;
+    auto failed = [&](cudaError_t e) -> cs_status {
+        set_last_error("mlp gradient", e);
+        cleanup();
+        return CS_ERR_CUDA;
+    };
+    cudaError_t e;
+    if ((e = cudaMemcpy(X, x, (size_t)B * 12, cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = cudaMemcpy(T, t, (size_t)B * 12, cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = cudaMemcpy(p, params, kNParams * 4, cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = cudaMemset(g, 0, kNParams * 4)) != cudaSuccess || (e = cudaMemset(w.loss, 0, 4)) != cudaSuccess)
+        return failed(e);
     if (fused) {
         StepArgs sa = {};
         ReduceArgs ra = {};
@@ -1131,16 +1136,23 @@ extern "C" cs_status cs_mlp_loss_grad(const float* params, const float* x, const
         sa.p = p;
         ra.g = g;
         ra.loss_out = w.loss;
-        if ((e = step_attributes()) == cudaSuccess) step_launch(sa, ra, nullptr);
+        if ((e = step_attributes()) != cudaSuccess) return failed(e);
+        step_launch(sa, ra, nullptr);
     } else {
         round_weights_kernel<<<(kNParams + 255) / 256, 256>>>(p, pr);
         forward(X, B, pr, w, nullptr);
         backward(X, T, nullptr, B, pr, g, w, nullptr);
     }
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    if (e != cudaSuccess) { set_last_error("mlp gradient", e); cleanup(); return CS_ERR_CUDA; }
-    cudaMemcpy(grad, g, kNParams * 4, cudaMemcpyDeviceToHost);
-    if (loss) cudaMemcpy(loss, w.loss, 4, cudaMemcpyDeviceToHost);
+    // a block whose wait gave up leaves its partial sums unwritten: no gradients
+    bool timed_out = false;
+    if ((e = cudaGetLastError()) != cudaSuccess || (e = tc_read_timeout(timed_out, nullptr)) != cudaSuccess) return failed(e);
+    if (timed_out) {
+        cleanup();
+        return CS_ERR_TIMEOUT;
+    }
+    if ((e = cudaMemcpy(grad, g, kNParams * 4, cudaMemcpyDeviceToHost)) != cudaSuccess ||
+        (loss && (e = cudaMemcpy(loss, w.loss, 4, cudaMemcpyDeviceToHost)) != cudaSuccess))
+        return failed(e);
     cleanup();
     return CS_OK;
 }
