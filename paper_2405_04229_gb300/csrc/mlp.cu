@@ -769,20 +769,27 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
     SurrogateView bv;
     memset(&bv, 0, sizeof bv);
     float4* d_base = nullptr;
+    cudaError_t e = cudaSuccess;
+    auto failed = [&](const char* where, cudaError_t err) -> cs_status {
+        set_last_error(where, err);
+        cudaFree(d_base);
+        cleanup();
+        return CS_ERR_CUDA;
+    };
     {
         std::vector<double> hb(kBaseN);
         for (int j = 0; j < kBaseN; ++j) hb[j] = cfg.h_min + (cfg.h_max - cfg.h_min) * j / (kBaseN - 1);
         double* d_hb = (double*)A(kBaseN * sizeof(double));
         Fields4* d_col = (Fields4*)A(kBaseN * sizeof(Fields4));
         if (!d_hb || !d_col || alloc((void**)&d_base, kBaseN * sizeof(float4)) != CS_OK) { cleanup(); return CS_ERR_CUDA; }
-        cudaMemcpy(d_hb, hb.data(), kBaseN * sizeof(double), cudaMemcpyHostToDevice);
+        if ((e = cudaMemcpy(d_hb, hb.data(), kBaseN * sizeof(double), cudaMemcpyHostToDevice)) != cudaSuccess) return failed("baseline", e);
         if ((st = column_fields(atm, d_hb, kBaseN, d_col, s)) != CS_OK) { cudaFree(d_base); cleanup(); return st; }
         std::vector<Fields4> col(kBaseN);
         std::vector<float4> tab(kBaseN);
-        cudaMemcpy(col.data(), d_col, kBaseN * sizeof(Fields4), cudaMemcpyDeviceToHost);
+        if ((e = cudaMemcpy(col.data(), d_col, kBaseN * sizeof(Fields4), cudaMemcpyDeviceToHost)) != cudaSuccess) return failed("baseline", e);
         for (int j = 0; j < kBaseN; ++j)
             tab[j] = make_float4((float)col[j].x, (float)col[j].y, (float)col[j].z, (float)col[j].w);
-        cudaMemcpy(d_base, tab.data(), kBaseN * sizeof(float4), cudaMemcpyHostToDevice);
+        if ((e = cudaMemcpy(d_base, tab.data(), kBaseN * sizeof(float4), cudaMemcpyHostToDevice)) != cudaSuccess) return failed("baseline", e);
         bv.base = d_base;
         bv.base_n = kBaseN;
         bv.base_dz0 = (float)(cfg.h_min - atm->p.h_obs);
@@ -800,8 +807,7 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
     baseline_kernel<<<base_blocks, kBaseThreads, 0, s>>>(bv, hth, lam, lab, Tphys, n_all, nt, atm->p.h_obs, b3, d_range);
     // output normalisation from the training targets (fields less baseline)
     std::vector<double> range((size_t)base_blocks * 6);
-    cudaError_t e = cudaMemcpy(range.data(), d_range, range.size() * sizeof(double), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) { set_last_error("labels", e); cudaFree(d_base); cleanup(); return CS_ERR_CUDA; }
+    if ((e = cudaMemcpy(range.data(), d_range, range.size() * sizeof(double), cudaMemcpyDeviceToHost)) != cudaSuccess) return failed("labels", e);
     double mn[3] = {1e300, 1e300, 1e300}, mx[3] = {-1e300, -1e300, -1e300};
     for (size_t b = 0; b < base_blocks; ++b) {
         for (int k = 0; k < 3; ++k) {
@@ -836,9 +842,9 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
         init(kOffW3, kHid, kHid, kHid);
         init(kOffW4, kNOutP, kHid, kNOut);
     }
-    cudaMemcpy(p, hp.data(), kNParams * 4, cudaMemcpyHostToDevice);
-    cudaMemset(m, 0, kNParams * 4);
-    cudaMemset(v, 0, kNParams * 4);
+    if ((e = cudaMemcpy(p, hp.data(), kNParams * 4, cudaMemcpyHostToDevice)) != cudaSuccess ||
+        (e = cudaMemset(m, 0, kNParams * 4)) != cudaSuccess || (e = cudaMemset(v, 0, kNParams * 4)) != cudaSuccess)
+        return failed("initial parameters", e);
     // ---- training -----------------------------------------------------------
     // A training step is ~20 short launches (the GEMMs of a 32768-row batch take microseconds), so
     // the steps run as captured CUDA graphs: the step's draws, learning rate and bias corrections
@@ -856,15 +862,10 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
         float4* sched = (float4*)A(hs.size() * sizeof(float4));
         unsigned int* step_ctr = (unsigned int*)A(2 * sizeof(unsigned int));   // and the fused reduction's own
         if (!sched || !step_ctr) { cudaFree(d_base); cleanup(); return CS_ERR_CUDA; }
-        cudaMemcpy(sched, hs.data(), hs.size() * sizeof(float4), cudaMemcpyHostToDevice);
-        cudaMemset(step_ctr, 0, 2 * sizeof(unsigned int));
-        if (fused) e = step_attributes();
-        if (e != cudaSuccess || (e = cudaDeviceSynchronize()) != cudaSuccess) {
-            set_last_error("surrogate training set-up", e);
-            cudaFree(d_base);
-            cleanup();
-            return CS_ERR_CUDA;
-        }
+        if ((e = cudaMemcpy(sched, hs.data(), hs.size() * sizeof(float4), cudaMemcpyHostToDevice)) != cudaSuccess ||
+            (e = cudaMemset(step_ctr, 0, 2 * sizeof(unsigned int))) != cudaSuccess ||
+            (fused && (e = step_attributes()) != cudaSuccess) || (e = cudaDeviceSynchronize()) != cudaSuccess)
+            return failed("surrogate training set-up", e);
         cudaStream_t ts = nullptr;
         cudaGraph_t graphs[2] = {nullptr, nullptr};
         cudaGraphExec_t execs[2] = {nullptr, nullptr};
@@ -932,12 +933,8 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
         }
         if (ts) cudaStreamDestroy(ts);
     }
-    if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess || (e = cudaDeviceSynchronize()) != cudaSuccess) {
-        set_last_error("surrogate training", e);
-        cudaFree(d_base);
-        cleanup();
-        return CS_ERR_CUDA;
-    }
+    if (e != cudaSuccess || (e = cudaGetLastError()) != cudaSuccess || (e = cudaDeviceSynchronize()) != cudaSuccess)
+        return failed("surrogate training", e);
     // ---- the trained network ---------------------------------------------------
     cs_surrogate* sg = new cs_surrogate;
     sg->d_base = d_base;
@@ -952,7 +949,15 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
     to_bf16_kernel<<<(kNBf16 + 255) / 256, 256, 0, s>>>(p, sg->d_wb);
     SurrogateNet& sv = sg->view;
     static_cast<SurrogateView&>(sv) = bv;   // the baseline table and constants
-    e = cudaMemcpy(hp.data(), p, kNParams * 4, cudaMemcpyDeviceToHost);
+    auto failed_net = [&](cudaError_t err) -> cs_status {
+        set_last_error("surrogate evaluation", err);
+        cleanup();
+        cs_surrogate_destroy(sg);   // (d_base is its own by now)
+        return CS_ERR_CUDA;
+    };
+    if ((e = cudaGetLastError()) != cudaSuccess ||
+        (e = cudaMemcpy(hp.data(), p, kNParams * 4, cudaMemcpyDeviceToHost)) != cudaSuccess)
+        return failed_net(e);
     for (int i = 0; i < kHid / 2; ++i) {
         const float *w = hp.data() + kOffW1 + 6 * i, *b = hp.data() + kOffB1 + 2 * i;
         sv.w1p[i][0] = make_float4(w[0], w[3], w[1], w[4]);
@@ -989,10 +994,11 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
     std::vector<Fields4> hl(nh);
     std::vector<double2> hhth(nh);
     std::vector<double> hlam(nh), Tp(nh);
-    cudaMemcpy(hl.data(), lab + nt, nh * sizeof(Fields4), cudaMemcpyDeviceToHost);
-    cudaMemcpy(hhth.data(), hth + nt, nh * sizeof(double2), cudaMemcpyDeviceToHost);
-    cudaMemcpy(hlam.data(), lam + nt, nh * sizeof(double), cudaMemcpyDeviceToHost);
-    cudaMemcpy(Tp.data(), Tphys + nt, nh * sizeof(double), cudaMemcpyDeviceToHost);
+    if ((e = cudaMemcpy(hl.data(), lab + nt, nh * sizeof(Fields4), cudaMemcpyDeviceToHost)) != cudaSuccess ||
+        (e = cudaMemcpy(hhth.data(), hth + nt, nh * sizeof(double2), cudaMemcpyDeviceToHost)) != cudaSuccess ||
+        (e = cudaMemcpy(hlam.data(), lam + nt, nh * sizeof(double), cudaMemcpyDeviceToHost)) != cudaSuccess ||
+        (e = cudaMemcpy(Tp.data(), Tphys + nt, nh * sizeof(double), cudaMemcpyDeviceToHost)) != cudaSuccess)
+        return failed_net(e);
     std::vector<float4> hin(nh);
     for (size_t i = 0; i < nh; ++i) {
         const double2 a = hhth[i];
@@ -1000,16 +1006,15 @@ extern "C" cs_status cs_surrogate_train(const cs_atmosphere* atm, const cs_surro
     }
     float4 *din = (float4*)A(nh * sizeof(float4)), *dout = (float4*)A(nh * sizeof(float4));
     std::vector<float4> hout(nh);
-    if (din && dout) {
-        cudaMemcpy(din, hin.data(), nh * sizeof(float4), cudaMemcpyHostToDevice);
-        const cs_status ev = run_eval(sv, din, nh, dout, s);
-        if (ev != CS_OK) {
-            cleanup();
-            cs_surrogate_destroy(sg);
-            return ev;
-        }
-        cudaMemcpy(hout.data(), dout, nh * sizeof(float4), cudaMemcpyDeviceToHost);
+    if (!din || !dout) return failed_net(cudaErrorMemoryAllocation);
+    if ((e = cudaMemcpy(din, hin.data(), nh * sizeof(float4), cudaMemcpyHostToDevice)) != cudaSuccess) return failed_net(e);
+    const cs_status ev = run_eval(sv, din, nh, dout, s);
+    if (ev != CS_OK) {
+        cleanup();
+        cs_surrogate_destroy(sg);
+        return ev;
     }
+    if ((e = cudaMemcpy(hout.data(), dout, nh * sizeof(float4), cudaMemcpyDeviceToHost)) != cudaSuccess) return failed_net(e);
     std::vector<double> er[3];
     for (size_t i = 0; i < nh; ++i) {
         const double th = hhth[i].y, c = cos(th), sn = sin(th);
