@@ -8,6 +8,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "exact_path.cuh"
@@ -399,7 +400,10 @@ extern "C" cs_status cs_atmosphere_create(const cs_atmosphere_desc* d, cs_atmosp
     a.R = d->earth_radius > 0.0 ? d->earth_radius : 6370000.0;
     if (d->geometry != CS_GEOM_PLANAR && d->geometry != CS_GEOM_SPHERICAL && d->geometry != CS_GEOM_CYLINDRICAL)
         return CS_ERR_INVALID_ARG;
-    a.H_A = d->aer_H > 0.0 ? d->aer_H : 1200.0;
+    // The FP64 points multiply by reciprocals of the scale heights (div_known), which an infinite one
+    // and a denormal one do not have: held to a range beyond which exp(-h / H) is 1 or 0 anyway.
+    auto scale_height = [](double H) { return std::min(std::max(H, 1e-200), 1e200); };
+    a.H_A = scale_height(d->aer_H > 0.0 ? d->aer_H : 1200.0);
     double table_top;
     if (d->kind == CS_ATM_LAYERED) {
         if (d->n_layers < 1 || d->n_layers > kMaxLayers) return CS_ERR_INVALID_ARG;
@@ -409,8 +413,8 @@ extern "C" cs_status cs_atmosphere_create(const cs_atmosphere_desc* d, cs_atmosp
             a.lay_h[i] = d->layer_h[i];
             a.lay_a[i] = d->layer_a[i];
             a.lay_b[i] = d->layer_b[i];
-            a.lay_c[i] = d->layer_c[i];
-            if (!(a.lay_c[i] > 0.0) || !(a.lay_b[i] > 0.0)) return CS_ERR_INVALID_ARG;
+            if (!(d->layer_c[i] > 0.0) || !(a.lay_b[i] > 0.0)) return CS_ERR_INVALID_ARG;
+            a.lay_c[i] = scale_height(d->layer_c[i]);
             if (i > 0 && !(a.lay_h[i] > a.lay_h[i - 1])) return CS_ERR_INVALID_ARG;
         }
         a.h_top = d->h_top;
