@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "exact_path.cuh"
+#include "known_divisor.cuh"
 
 namespace cs {
 namespace {
@@ -80,13 +81,6 @@ __device__ inline void delta_rho(const AtmF64& a, double h, bool below, double* 
         *rho = 0.0;
         *delta = a.hom_delta;
     }
-}
-
-// x / c for rc = 1 / c correctly rounded (Markstein, "Computation of elementary functions on the IBM
-// RISC System/6000", 1990): the remainder of the first quotient, exact through FMA, corrects it.
-__device__ inline double div_known(double x, double c, double rc) {
-    const double q = x * rc;
-    return fma(fma(-q, c, x), rc, q);
 }
 
 // Breakpoints of n(h) strictly inside (h_obs, h_e), between h_obs and h_e; returns their number.
@@ -201,7 +195,6 @@ __device__ void node_fields(const AtmF64& a, const PieceTable& tab, double h_e, 
             if (a.refraction) {
                 const double q = sqrt(n * n - s * s), rq = 1.0 / q;
                 acc[0] += wt * (de - d) * (2.0 + de + d) / (q * fma(ne, cos0, q));
-
                 acc[1] += div_known(wt * (n * n * cos0 - q), q, rq);
                 acc[2] += div_known(wt * 100.0 * rho * n, q, rq);
                 acc[3] += div_known(wt * ea * n, q, rq);
