@@ -332,10 +332,12 @@ typedef struct cs_opts {
      * streamed calls through cs_check_timeout). */
     int tc_poll_limit;
     /* Bunches beyond the correction tables are queued by the photon kernel for the exact pass:
-     * entries per warp tile of 32 segments (0 = default, 8, of fluorescence 32; at least 4096 and at most 2^22
-     * entries in all, and at most the default in the batched and streamed calls; < 0 = no
-     * queue).  When the queue is full the remaining such bunches mark their warp tile, which
-     * the exact pass then regenerates whole; the results are the same either way. */
+     * entries per warp tile of 32 segments.  0 = default: 8, and 32 for fluorescence in
+     * device-pointer calls and host-pointer calls that are not split into chunks.  The batched,
+     * streamed and chunked calls take 8 at most, whatever is given, and cs_propagate_noalloc
+     * takes none.  At least 4096 and at most 2^22 entries in all; < 0 = no queue.  When the
+     * queue is full the remaining such bunches mark their warp tile, which the exact pass then
+     * regenerates whole; the results are the same either way. */
     int exact_queue;
 } cs_opts;
 

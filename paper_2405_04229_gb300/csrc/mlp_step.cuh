@@ -13,7 +13,9 @@
 //
 // Arithmetic and its order are the unfused path's: the same BF16 hi + lo
 // splits, the same K = 16 products in the same order, partial sums over the
-// same rows, so both give the same bits.
+// same rows.  Loss and gradients of 256, 512, 4,352, 32,768, 33,024 and
+// 131,072 rows were equal bit for bit to those of the library from before
+// this step, which took these sizes through global memory.
 //
 // Operand tiles: an activation tile of 128 rows x 64 units is stored once, in
 // the no-swizzle core-matrix layout with the units contiguous.  As the A
@@ -409,7 +411,7 @@ struct ReduceArgs {
 // of the other partial sums by 128 threads and a pairwise tree; one block per 32 weight elements,
 // then one per column.  The 9 MB of slices of a 32,768-row batch come from L2 through shared memory,
 // 256 slices at a time by all threads, so that the loads and not the serial sum set the pace
-// (one thread per element loading its own slices took 24 us, this form 14 us).
+// (one thread per element loading its own slices took 24 us, this form 11 us with the slices in L2).
 constexpr int kRedThreads = 128, kRedW = 2 * kHid * kHid + kNOutP * kHid, kRedWPer = 32;
 constexpr int kRedCols = 3 * kHid + kHid * kNIn + 1 + kNOut;
 constexpr int kRedBlocks = kRedW / kRedWPer + kRedCols;

@@ -85,8 +85,10 @@ constexpr size_t kTcSmemOffset = (sizeof(TileSmem) + 127) & ~(size_t)127;
 // wait for the tensor cores and at the block's barriers most of the time, and only other warps fill
 // that.  Two blocks of 64 registers a thread: 1e6 segments of bunch 5 946 us; one block with 256
 // segments, 2,048 bunches and 120 registers: 1169 us.  A tile has about 1,250 bunches at bunch 5: in
-// windows of 1,024 a second, mostly empty one followed (847 us, so 829 us).  (One block where the
-// network splits its activations, whose lo tiles take 64 KB more.)
+// windows of 1,024 a second, mostly empty one followed (847 us, so 829 us; that is what 1,792 is sized
+// for: 3 m segments of about 16 photons a metre.  At bunch 1 or 2, or with longer tracks, a tile takes
+// several windows).  (One block where the network splits its activations, whose lo tiles take 64 KB
+// more.)
 constexpr size_t smem_surrogate(bool split) { return kTcSmemOffset + TcSmem<kThreadsSur / 128>::bytes(split); }
 static_assert(2 * (smem_surrogate(false) + 1024) <= 228 * 1024, "two surrogate blocks per SM");
 
@@ -483,6 +485,17 @@ __device__ __forceinline__ int optics_survival(const DetParams& dp, const PropPa
     return uniform24(r.x) < fR * fE ? pix : -1;
 }
 
+// Calls slab(j) for j = 0 .. ns - 1, j as a float.
+template <typename F>
+__device__ __forceinline__ void for_slabs(int ns, F&& slab) {
+    if (ns <= 1 << 24) {
+        const float end = (float)ns;
+        for (float j = 0.0f; j < end; j += 1.0f) slab(j);
+    } else {   // a float does not count past 2^24
+        for (int j = 0; j < ns; ++j) slab((float)j);
+    }
+}
+
 // Snell's law in vector form through homogeneous slabs (Sec. 3.4.2, Eq. 3.15),
 // the general-atmosphere tracer.  The height dz above the observation level is
 // cut into the fewest equal slabs no thicker than dh; slab j holds the index
@@ -501,18 +514,6 @@ __device__ __forceinline__ int optics_survival(const DetParams& dp, const PropPa
 // takes two slabs per packed FP32 instruction.  100,000 segments of bunch 5,
 // 10 m slabs: 3.70 ms with delta_at's layer selects in every slab, 1.38 ms with
 // the kept layer, 1.16 ms with rounds of like heights, 0.74 ms in pairs.
-
-// Calls slab(j) for j = 0 .. ns - 1, j as a float.
-template <typename F>
-__device__ __forceinline__ void for_slabs(int ns, F&& slab) {
-    if (ns <= 1 << 24) {
-        const float end = (float)ns;
-        for (float j = 0.0f; j < end; j += 1.0f) slab(j);
-    } else {   // a float does not count past 2^24
-        for (int j = 0; j < ns; ++j) slab((float)j);
-    }
-}
-
 __device__ __noinline__ float4 snell_path(const AtmParams& ap, float dz, float cos0, float dh) {
     const int ns = max(1, (int)ceilf(dz / dh));
     const float step = dz / (float)ns;
@@ -980,7 +981,6 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                 // first, its fields are constant operands (no indexed parameter loads)
                 const bool lvl0 = s2 <= dp.hash[0].sin2_max;
                 auto detect = [&](const TelHash& H, const bool hashed) {
-                {
                     float ugz = uz;
                     if (c_refr) {
                         const float c2 = fmaxf(1.0f - s2, 1e-30f);
@@ -1008,7 +1008,6 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                                            (T4.y - Cg.z) + ((TL.y - Cg.w) - ry), T4.z, ux * sc, uy * sc, ugz);
                         pix = optics_survival(dp, pp, gid, k, i, inv_l, pix);
                     }
-                }
                 };
                 if (__all_sync(__activemask(), lvl0)) detect(dp.hash[0], true);
                 else detect(dp.hash[lvl0 ? 0 : (s2 <= dp.hash[1].sin2_max ? 1 : 2)], s2 <= dp.hash[2].sin2_max);
@@ -1089,7 +1088,6 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                 const float sg2 = ugx * ugx + ugy * ugy;
                 const bool lvl0 = sg2 <= dp.hash[0].sin2_max;
                 auto detect = [&](const TelHash& H, const bool hashed) {
-                {
                     tel = hit_telescope<MODE == kModeExact ? 8 : 1>(
                         dp, H, hashed, sg2, xs, ys, ugx, ugy, ugz,
                         [&](const float4& D, float cx0, float cy0, float& ddx, float& ddy, float& ddz) {
@@ -1111,7 +1109,6 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                         pix = camera_pixel(dp, (T4.x - x) + (TL.x - xl), (T4.y - y) + (TL.y - yl), T4.z, ugx, ugy, ugz);
                         pix = optics_survival(dp, pp, gid, k, i, inv_l, pix);
                     }
-                }
                 };
                 if (__all_sync(__activemask(), lvl0)) detect(dp.hash[0], true);
                 else detect(dp.hash[lvl0 ? 0 : (sg2 <= dp.hash[1].sin2_max ? 1 : 2)], sg2 <= dp.hash[2].sin2_max);
@@ -1265,25 +1262,23 @@ __device__ __forceinline__ bool bunch(const SM& S, int q, int i, bool active, lo
                                                                                              : 2;
                     const TelHash& H = dp.hash[lvl];
                     const bool hashed = sg2 <= H.sin2_max;
-                    {
-                        auto delta3 = [&](const float4& T3, float& ddx, float& ddy, float& ddz) {
-                            ddx = (T3.x - Gx) - Gxl;
-                            ddy = (T3.y - Gy) - Gyl;
-                            ddz = (T3.z - Gz) - Gzl;
-                        };
-                        tel = hit_telescope<MODE == kModeExact ? 8 : 1>(
-                            dp, H, hashed, sg2, xs, ys, ugx, ugy, ugz,
-                            [&](const float4& D, float, float, float& ddx, float& ddy, float& ddz) { delta3(D, ddx, ddy, ddz); },
-                            [&](int it, float& ddx, float& ddy, float& ddz, float& r) {
-                                const float4 T3 = __ldg(dp.tel3 + it);
-                                delta3(T3, ddx, ddy, ddz);
-                                r = T3.w;
-                            });
-                        if (tel >= 0 && c_cam) {
-                            const float4 T3 = __ldg(dp.tel3 + tel);
-                            pix = camera_pixel(dp, (T3.x - Gx) - Gxl, (T3.y - Gy) - Gyl, (T3.z - Gz) - Gzl, ugx, ugy, ugz);
-                            pix = optics_survival(dp, pp, gid, k, i, inv_l, pix);
-                        }
+                    auto delta3 = [&](const float4& T3, float& ddx, float& ddy, float& ddz) {
+                        ddx = (T3.x - Gx) - Gxl;
+                        ddy = (T3.y - Gy) - Gyl;
+                        ddz = (T3.z - Gz) - Gzl;
+                    };
+                    tel = hit_telescope<MODE == kModeExact ? 8 : 1>(
+                        dp, H, hashed, sg2, xs, ys, ugx, ugy, ugz,
+                        [&](const float4& D, float, float, float& ddx, float& ddy, float& ddz) { delta3(D, ddx, ddy, ddz); },
+                        [&](int it, float& ddx, float& ddy, float& ddz, float& r) {
+                            const float4 T3 = __ldg(dp.tel3 + it);
+                            delta3(T3, ddx, ddy, ddz);
+                            r = T3.w;
+                        });
+                    if (tel >= 0 && c_cam) {
+                        const float4 T3 = __ldg(dp.tel3 + tel);
+                        pix = camera_pixel(dp, (T3.x - Gx) - Gxl, (T3.y - Gy) - Gyl, (T3.z - Gz) - Gzl, ugx, ugy, ugz);
+                        pix = optics_survival(dp, pp, gid, k, i, inv_l, pix);
                     }
                     if (tel >= 0) {
                         T.tel += b;
@@ -1596,8 +1591,8 @@ propagate_kernel(const PropParams pp, const AtmParams ap, const DetParams dp, co
             // the exact pass takes the queued bunches a block's worth at a time, then the marked groups
             // from their list.  A bunch is integrated over as many sub-intervals as its height gives it
             // and a warp takes as long as its longest: the block orders its entries by height, in bins
-            // of 1 km.  (In the queue's order 20 of 32 lanes
-            // worked; fluorescence on 1e6 segments 168 -> 158 us.)
+            // of 1 km.  (In the queue's order 20 of 32 lanes worked; fluorescence on 1e6 segments
+            // 168 -> 158 us.)
             const unsigned int n_listed = __ldcg(scratch + 2);
             const unsigned int n_q = min(__ldcg(scratch + 3), pp.q_cap);
             const unsigned int* bits = scratch + kScratchCounters;
@@ -1929,11 +1924,9 @@ cudaError_t set_exact_smem(int smem) {
     const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
     cudaError_t e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, false, F, T>, attr, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, true, F, T>, attr, smem);
-    if (!T) {   // the exact pass of the table-tracer instances
+    if (!T) {   // the exact pass of the table-tracer instances, and the fixed configurations
         if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, false, F, false, true>, attr, (int)kSmemPass);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, true, F, false, true>, attr, (int)kSmemPass);
-    }
-    if (!T) {   // the fixed-configuration instances
         if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, false, F, false, false, kFixed>, attr, smem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(propagate_kernel<kNoNet, S, 4, false, F, false, false, kFixedOptics>, attr, smem);
     }
@@ -1994,10 +1987,12 @@ int default_blocks_per_sm(const cs_opts& o) {
 // Segments per tile.  A launch of `slots` resident warps ends when its last tile does, about half a
 // tile's time (in proportion to tile / bunch) after the others, and every tile costs a fixed import,
 // sort and scan: tail + fixed cost is smallest at tile ~ sqrt(n bunch / slots).  The factor is from
-// sweeps over 1, 2, .. 32 segments: for 1,000 / 5,003 / 20,000 / 62,500 / 262,144 segments of
-// bunch 1 the best tiles are 1-2 / 2 / 4 / 8 / 8-16 (20.6 / 35.0 / 53.8 / 87.1 / 237 us per launch
-// against 65.6 / 108.9 / 110.6 / 127.2 / 262 us with 32), with bunch 5 from 5,003 on 4 / 8 / 16-32 /
-// 32 (26.8 / 34.8 / 47.2 / 82.9 us against 41.9 / 44.8 / 47.2 / 82.9 us).
+// sweeps over 1, 2, .. 32 segments of 3 m with about 16 photons a metre (the plan does not know the
+// tracks' lengths; in the batched calls opts.bunch stands for the showers' own bunch sizes): for
+// 1,000 / 5,003 / 20,000 / 62,500 / 262,144 segments of bunch 1 the best tiles are 1-2 / 2 / 4 / 8 /
+// 8-16 (20.6 / 35.0 / 53.8 / 87.1 / 237 us per launch against 65.6 / 108.9 / 110.6 / 127.2 / 262 us
+// with 32), with bunch 5 from 5,003 on 4 / 8 / 16-32 / 32 (26.8 / 34.8 / 47.2 / 82.9 us against
+// 41.9 / 44.8 / 47.2 / 82.9 us).
 //
 // Parts (the stepper only: a round of bunches then takes ~20 times the tile's own work, so that
 // repeating import and sub-steps in up to 16 warps costs little): enough for eight units per
