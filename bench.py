@@ -82,6 +82,12 @@ def workload(seed, n_showers=10, per_shower=100_000):
     return segs, synth.grid_telescopes(), synth.histogram_400()
 
 
+def ground(rec):
+    """Ground points of records in FP64: the sums of their float pairs (on the sphere the
+    second part holds the whole refraction correction)."""
+    return tuple(rec[k].astype(np.float64) + rec[k + "_lo"] for k in ("x", "y"))
+
+
 def substeps(segs, s_max=1.0):
     L = segs["length"].astype(np.float32)
     return int(np.maximum(1, np.ceil(L / np.float32(s_max))).sum())
@@ -491,9 +497,10 @@ def run_inclined(args):
         ra, rb = recs[0][ia], recs[1][ib]
         both = np.isin(ra["status"], [B.CS_ST_LANDED, B.CS_ST_ABSORBED]) & \
             np.isin(rb["status"], [B.CS_ST_LANDED, B.CS_ST_ABSORBED])
-        shift = float(np.hypot(ra["x"].astype(np.float64) - rb["x"], ra["y"].astype(np.float64) - rb["y"])[both].max())
+        (xa, ya), (xb, yb) = ground(ra), ground(rb)
+        shift = float(np.hypot(xa - xb, ya - yb)[both].max())
         radius, margin = 1000.0 * math.sqrt(2.0) + 6.0, 1.5 * shift + 1.0
-        straight = np.hypot(rb["x"].astype(np.float64), rb["y"].astype(np.float64))
+        straight = np.hypot(xb, yb)
         B.set_lv3(o, dict(centre=(0.0, 0.0, 2000.0), radius=radius, margin=margin))
         step()
         torch.cuda.synchronize()
